@@ -5,7 +5,9 @@
 // the FFT twiddles, the pair-tile schedule over the N(N+1)/2 pairs (Sec. 2,
 // pair-count paragraph; Table pscount) and the device workspace of one tile.
 // exx_apply / exx_energy enqueue the tile pipeline behind the caller's stream:
-//   fwd_xy -> zconv -> pair_energy [-> inv_yx -> accum]   per pair tile
+//   xfwd -> plane -> pair_energy [-> xinv -> accum]   per pair tile
+//   (fwd_xy -> zconv -> pair_energy [-> inv_yx -> accum] where the plane
+//   pipeline is not built: Ops::plane_ok)
 //   exx_total [-> convert]                                once
 // With two or three lanes the transforms of consecutive tiles run on the
 // lanes' internal streams (forked from and joined back into the caller's
@@ -231,6 +233,9 @@ struct exx_plan_s {
   double h = 0.0, alpha = 0.0, omega = 0.0;
   std::vector<double> occ;
   const Ops* ops = nullptr;
+  bool plane = false;  // plane pipeline (exx_plane.cuh)
+  size_t y_off = 0;    // byte offset of its second spectrum buffer in X2 (plane_ry = 2), else 0
+  int nper = 0;        // energy partials per pair
   int T = 0;
   std::vector<Tile> tiles;
   std::vector<char> mine;  // tiles this plan processes (all unless sharded)
@@ -518,16 +523,27 @@ static exx_status_t plan_create_impl(exx_plan_t* out, const int grid[3], const d
   const size_t cs = 2 * rs;
   // kernel table (scaled by 1/(L^2 LZ); for FP32 with the forward transforms'
   // gains divided out) and twiddle tables (exx_ops.cuh)
-  std::vector<unsigned char> gbuf(exx::kernel_table_bytes(nh, nz, rs, ops->table_fold_y)),
-      twbuf(exx::twiddle_count(nh) * cs), twzbuf(nz != nh ? exx::twiddle_count(nz) * cs : 0);
+  p->plane = ops->plane_ok;
+  const bool sep_z = nz != nh && !p->plane;  // z twiddles of their own
+  std::vector<unsigned char> gbuf(exx::kernel_table_bytes(nh, nz, rs, ops->table_fold_y && !p->plane)),
+      twbuf((p->plane ? ops->plane_twiddles : exx::twiddle_count(nh)) * cs),
+      twzbuf(sep_z ? exx::twiddle_count(nz) * cs : 0);
   std::vector<double> gx, gy, gz;
   if (ops->gains) {
     gx.resize(m);
     gy.resize(2 * (size_t)nh);
     gz.resize(2 * (size_t)nz);
-    ops->gains(gx.data(), gy.data(), gz.data());
+    (p->plane ? ops->plane_gains : ops->gains)(gx.data(), gy.data(), gz.data());
   }
-  if (precision == EXX_FP64) {
+  if (p->plane) {
+    const double *ax = gx.empty() ? nullptr : gx.data(), *ay = gx.empty() ? nullptr : gy.data(),
+                 *az = gx.empty() ? nullptr : gz.data();
+    if (precision == EXX_FP64)
+      exx::build_plane_table<double>(nh, nz, ops->plane_ry, Gh.data(), scale, ax, ay, az, gbuf.data());
+    else
+      exx::build_plane_table<float>(nh, nz, ops->plane_ry, Gh.data(), scale, ax, ay, az, gbuf.data());
+    ops->plane_build_twiddles(twbuf.data());
+  } else if (precision == EXX_FP64) {
     exx::build_kernel_table<double>(nh, nz, ops->table_fold_y, Gh.data(), scale, nullptr, nullptr,
                                     nullptr, gbuf.data());
     exx::build_twiddles(nh, reinterpret_cast<double*>(twbuf.data()));
@@ -542,7 +558,16 @@ static exx_status_t plan_create_impl(exx_plan_t* out, const int grid[3], const d
   }
 
   const long long n3 = (long long)n * n * n;
-  const size_t nper = m * (size_t)ops->nyb;
+  const size_t nper = m * (size_t)(p->plane ? ops->plane_ne : ops->nyb);
+  p->nper = (int)nper;
+  // spectra of one tile: padded along y, or the plane pipeline's unpadded ones
+  // (two buffers where its planes go through in two halves)
+  size_t xbytes = (size_t)p->maxpairs * m * n * (2 * nh) * cs;
+  if (p->plane) {
+    const size_t one = (size_t)p->maxpairs * m * n * n * cs;
+    p->y_off = ops->plane_ry == 2 ? one : 0;
+    xbytes = one * ops->plane_ry;
+  }
   exx_status_t st_;
   // test hook (EXX_TEST_FAIL_ALLOC=k, k >= 1): the plan's k-th device
   // allocation reports out of memory without calling cudaMalloc, so that the
@@ -566,26 +591,26 @@ static exx_status_t plan_create_impl(exx_plan_t* out, const int grid[3], const d
   EXX_ALLOC(p->d_pairs, pairs.size() * sizeof(int4));
   EXX_ALLOC(p->epart, (size_t)p->maxpairs * nper * sizeof(double));
   EXX_ALLOC(p->Epair, (size_t)p->P * sizeof(double));
-  EXX_ALLOC(p->X2, (size_t)p->maxpairs * m * n * (2 * nh) * cs);
+  EXX_ALLOC(p->X2, xbytes);
   EXX_ALLOC(p->V, (size_t)p->maxpairs * n3 * rs);
   if (precision == EXX_FP32 && !(flags & EXX_FLAG_VX_FP64)) {
     EXX_ALLOC(p->vacc, (size_t)norb * n3 * sizeof(double));
   }
   EXX_ALLOC(p->E_dev, sizeof(double));
   EXX_ALLOC(p->d_err, 2 * sizeof(int));
-  // pipeline lanes: two by default, one where the slab kernels run as CTA
-  // clusters (512 orbitals on 160^3: 16.53 s per step with one lane, 16.59 s
-  // with two); EXX_LANES=1..3 at plan creation chooses; never more than the
+  // pipeline lanes: two by default (a tile's line kernels, bound by memory, run
+  // beside the other tile's plane kernel: 96^3 8.81 -> 8.50 ms with 32
+  // orbitals), one where the slab kernels run as CTA clusters; EXX_LANES=1..3 at plan creation chooses; never more than the
   // plan has tiles
   {
     const char* env = std::getenv("EXX_LANES");
-    int nl = ops->clustered ? 1 : kDefaultLanes;
+    int nl = ops->clustered && !p->plane ? 1 : kDefaultLanes;
     if (env && env[0] >= '1' && env[0] <= '0' + kMaxLanes && env[1] == '\0') nl = env[0] - '0';
     p->max_lanes = p->lanes = (int)std::min<size_t>((size_t)nl, p->tiles.size());
   }
   for (int l = 1; l < p->max_lanes; ++l) {
     EXX_ALLOC(p->epx[l], (size_t)p->maxpairs * nper * sizeof(double));
-    EXX_ALLOC(p->X2x[l], (size_t)p->maxpairs * m * n * (2 * nh) * cs);
+    EXX_ALLOC(p->X2x[l], xbytes);
     EXX_ALLOC(p->Vx[l], (size_t)p->maxpairs * n3 * rs);
   }
 #undef EXX_ALLOC
@@ -611,9 +636,9 @@ static exx_status_t plan_create_impl(exx_plan_t* out, const int grid[3], const d
     }
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess && ops->stage_table && !exx::make_ktab_map(&p->gmap, p->Gs, nh, nz))
+  if (e == cudaSuccess && ops->stage_table && !p->plane && !exx::make_ktab_map(&p->gmap, p->Gs, nh, nz))
     e = cudaErrorInvalidValue;
-  if (e == cudaSuccess) e = ops->setup();
+  if (e == cudaSuccess) e = p->plane ? ops->plane_setup() : ops->setup();
   if (e == cudaSuccess && p->max_lanes > 1) {
     for (int l = 0; l < p->max_lanes && e == cudaSuccess; ++l) {
       e = cudaStreamCreateWithFlags(&p->ls[l], cudaStreamNonBlocking);
@@ -672,7 +697,7 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
   const int n = p->n, N = p->N;
   const long long n3 = (long long)n * n * n;
   const double h3 = p->h * p->h * p->h;
-  const int nper = (p->ops->n + 1) * p->ops->nyb;
+  const int nper = p->nper;
   double* acc = nullptr;
   if (apply) {
     acc = p->vacc ? p->vacc : static_cast<double*>(vxpsi);
@@ -715,18 +740,20 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
     void* X2 = X2l[l];
     void* Vt = Vl[l];
     double* ep = epl[l];
+    void* Yt = static_cast<char*>(X2) + p->y_off;
     if (ov) {
       const int bj = t.j0 / p->T;
       while (waited[l] < bj) EXX_CUDA(p, cudaStreamWaitEvent(sl, (*ov->in)[++waited[l]], 0));
     }
     {
       ProfScope ps(p, K_FWD, sl);
-      p->ops->fwd_xy(psi, nullptr, pr, t.count, X2, p->tw, n3, sl);
+      if (p->plane) p->ops->xfwd(psi, nullptr, pr, t.count, X2, p->tw, n3, sl);
+      else p->ops->fwd_xy(psi, nullptr, pr, t.count, X2, p->tw, n3, sl);
     }
     {
       ProfScope ps(p, K_ZCONV, sl);
-      p->ops->zconv(X2, p->Gs, p->twz ? p->twz : p->tw, &p->gmap, ep, p->d_err, t.count, !apply,
-                    sl);
+      if (p->plane) p->ops->plane(X2, Yt, p->Gs, p->tw, ep, t.count, !apply, sl);
+      else p->ops->zconv(X2, p->Gs, p->twz ? p->twz : p->tw, &p->gmap, ep, p->d_err, t.count, !apply, sl);
     }
     {
       ProfScope ps(p, K_PAIRE, sl);
@@ -737,7 +764,8 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
       if (nl > 1 && used[l]) EXX_CUDA(p, cudaStreamWaitEvent(sl, p->ev_free[l], 0));
       {
         ProfScope ps(p, K_INV, sl);
-        p->ops->inv_yx(X2, Vt, p->tw, t.count, sl);
+        if (p->plane) p->ops->xinv(Yt, Vt, p->tw, t.count, sl);
+        else p->ops->inv_yx(X2, Vt, p->tw, t.count, sl);
       }
       if (nl > 1) {
         EXX_CUDA(p, cudaEventRecord(p->ev_done[l], sl));

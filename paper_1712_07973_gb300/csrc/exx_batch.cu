@@ -93,9 +93,13 @@ struct Group {
   const Ops* ops = nullptr;
   std::vector<int> mols;
   std::vector<Wave> waves;
-  void* Gs = nullptr;
+  bool plane = false;  // launch-per-pass schedule: the plane pipeline (exx_plane.cuh)
+  size_t one = 0;      // bytes of one spectrum buffer of the largest wave (plane)
+  void* Gs = nullptr;  // kernel table and twiddles of the launch-per-pass schedule
   void* tw = nullptr;
-  CUtensorMap gmap{};  // TMA descriptor of Gs (ops->stage_table)
+  CUtensorMap gmap{};  // TMA descriptor of Gs (ops->stage_table, slab pipeline)
+  void* Gs_q = nullptr;  // those of the persistent queue (the slab pipeline's layout),
+  void* tw_q = nullptr;  // built when it is first enabled
   // persistent mode: the group's queue segments (offset into the batch's
   // segment table and count, per mode: 0 apply or gradient, 1 energy), items,
   // and accumulation point blocks per tile
@@ -175,6 +179,8 @@ void batch_free(exx_batch_t b) {
   for (Group& g : b->groups) {
     if (g.Gs) cudaFree(g.Gs);
     if (g.tw) cudaFree(g.tw);
+    if (g.Gs_q) cudaFree(g.Gs_q);
+    if (g.tw_q) cudaFree(g.tw_q);
   }
   for (int k = 0; k < 3; ++k)
     if (b->gexec[k]) cudaGraphExecDestroy(b->gexec[k]);
@@ -313,8 +319,8 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
       a.V[1] = static_cast<float*>(b->V_2);
       a.epart[0] = b->epart;
       a.epart[1] = b->epart2;
-      a.Gs = static_cast<const float*>(g.Gs);
-      a.tw = static_cast<const float2*>(g.tw);
+      a.Gs = static_cast<const float*>(g.plane ? g.Gs_q : g.Gs);
+      a.tw = static_cast<const float2*>(g.plane ? g.tw_q : g.tw);
       a.Epair = b->Epair;
       a.vx_tab = b->d_vacc_tab;
       a.occ = b->d_occ;
@@ -329,21 +335,28 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
       if (g.ops->persist(a, st) != cudaSuccess) return EXX_ERR_CUDA;
       continue;
     }
-    const int nper = (g.n + 1) * g.ops->nyb;
+    const int nper = (g.n + 1) * (g.plane ? g.ops->plane_ne : g.ops->nyb);
     const double h3 = g.h * g.h * g.h;
     for (const Wave& w : g.waves) {
       const int4* pr = b->d_pairs + w.pair_off;
       const int l = nl > 1 ? (k++ & 1) : 0;
       cudaStream_t sl = nl > 1 ? b->ls[l] : st;
-      g.ops->fwd_xy(nullptr, reinterpret_cast<const void* const*>(b->d_psi_tab), pr, w.npair, Xl[l],
-                    g.tw, n3, sl);
-      g.ops->zconv(Xl[l], g.Gs, g.tw, &g.gmap, epl[l], b->d_err, w.npair, !apply, sl);
+      const void* const* psi_tab = reinterpret_cast<const void* const*>(b->d_psi_tab);
+      void* Yl = static_cast<char*>(Xl[l]) + (g.plane && g.ops->plane_ry == 2 ? g.one : 0);
+      if (g.plane) {
+        g.ops->xfwd(nullptr, psi_tab, pr, w.npair, Xl[l], g.tw, n3, sl);
+        g.ops->plane(Xl[l], Yl, g.Gs, g.tw, epl[l], w.npair, !apply, sl);
+      } else {
+        g.ops->fwd_xy(nullptr, psi_tab, pr, w.npair, Xl[l], g.tw, n3, sl);
+        g.ops->zconv(Xl[l], g.Gs, g.tw, &g.gmap, epl[l], b->d_err, w.npair, !apply, sl);
+      }
       k_pair_energy<<<(w.npair * 32 + 255) / 256, 256, 0, sl>>>(epl[l], nper, pr, w.npair, h3,
                                                                  b->Epair);
       if (apply) {
         if (nl > 1 && used[l] && cudaStreamWaitEvent(sl, b->ev_free[l], 0) != cudaSuccess)
           return EXX_ERR_CUDA;
-        g.ops->inv_yx(Xl[l], Vl[l], g.tw, w.npair, sl);
+        if (g.plane) g.ops->xinv(Yl, Vl[l], g.tw, w.npair, sl);
+        else g.ops->inv_yx(Xl[l], Vl[l], g.tw, w.npair, sl);
         if (nl > 1 && (cudaEventRecord(b->ev_done[l], sl) != cudaSuccess ||
                        cudaStreamWaitEvent(st, b->ev_done[l], 0) != cudaSuccess))
           return EXX_ERR_CUDA;
@@ -415,6 +428,37 @@ exx_status_t run_batch(exx_batch_t b, double* E_dev, bool apply, bool grad, cuda
   return cudaGraphLaunch(b->gexec[k], st) == cudaSuccess ? EXX_OK : EXX_ERR_CUDA;
 }
 
+// Kernel table and twiddles of a group, built on the host and copied (plane:
+// the plane pipeline's layout, else the slab pipeline's); synchronises st.
+exx_status_t group_tables(exx_batch_t b, const Group& g, bool plane, void** Gs, void** tw, cudaStream_t st) {
+  const Ops* ops = g.ops;
+  const size_t m = (size_t)g.n + 1;
+  std::vector<double> Gh(m * m * m);
+  if (!exx_host::kernel_spectrum_octant(g.n, g.h, g.kind, 0.0, Gh.data())) return EXX_ERR_INVALID_ARG;
+  const double L = 2.0 * g.n, scale = 1.0 / (L * L * L);
+  std::vector<double> gx(m), gy(2 * (size_t)g.n), gz(2 * (size_t)g.n);
+  (plane ? ops->plane_gains : ops->gains)(gx.data(), gy.data(), gz.data());
+  std::vector<unsigned char> gf(exx::kernel_table_bytes(g.n, g.n, sizeof(float), !plane && ops->table_fold_y));
+  std::vector<float> twf(2 * (plane ? ops->plane_twiddles : exx::twiddle_count(g.n)));
+  if (plane) {
+    exx::build_plane_table<float>(g.n, g.n, ops->plane_ry, Gh.data(), scale, gx.data(), gy.data(), gz.data(),
+                                  gf.data());
+    ops->plane_build_twiddles(twf.data());
+  } else {
+    exx::build_kernel_table<float>(g.n, g.n, ops->table_fold_y, Gh.data(), scale, gx.data(), gy.data(), gz.data(),
+                                   gf.data());
+    exx::build_twiddles(g.n, twf.data());
+  }
+  if (!balloc(b, Gs, gf.size()) || !balloc(b, tw, twf.size() * sizeof(float))) return EXX_ERR_OOM;
+  if (cudaMemcpyAsync(*Gs, gf.data(), gf.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      cudaMemcpyAsync(*tw, twf.data(), twf.size() * sizeof(float), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess) {  // the host buffers die here
+    cudaGetLastError();
+    return EXX_ERR_CUDA;
+  }
+  return EXX_OK;
+}
+
 int default_tile(int N, int requested) {
   int T = requested > 0 ? requested : 8;
   if (T > 8) T = 8;
@@ -471,6 +515,7 @@ exx_status_t exx_batch_create(exx_batch_t* out, int nmol, const exx_mol_desc* mo
       g.h = d.h;
       g.kind = kernel;
       g.ops = find_ops(EXX_FP32, d.n);
+      g.plane = g.ops->plane_ok;
       mm.group = (int)b->groups.size();
       b->groups.push_back(g);
     }
@@ -533,9 +578,10 @@ exx_status_t exx_batch_create(exx_batch_t* out, int nmol, const exx_mol_desc* mo
       g.waves.push_back(w);
       const size_t cs = sizeof(float2), rs = sizeof(float);
       const size_t n = (size_t)g.n;
-      b->x_bytes = std::max(b->x_bytes, (size_t)w.npair * (n + 1) * n * 2 * n * cs);
+      g.one = std::max(g.one, (size_t)w.npair * (n + 1) * n * n * cs);
+      b->x_bytes = std::max(b->x_bytes, g.one * (g.plane ? g.ops->plane_ry : 2));
       b->v_bytes = std::max(b->v_bytes, (size_t)w.npair * n * n * n * rs);
-      b->ep_bytes = std::max(b->ep_bytes, (size_t)w.npair * (n + 1) * g.ops->nyb * sizeof(double));
+      b->ep_bytes = std::max(b->ep_bytes, (size_t)w.npair * (n + 1) * std::max(g.ops->nyb, g.ops->plane_ne) * sizeof(double));
       b->max_wave_pairs = std::max(b->max_wave_pairs, w.npair);
     }
   }
@@ -578,32 +624,14 @@ exx_status_t exx_batch_create(exx_batch_t* out, int nmol, const exx_mol_desc* mo
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_vx_tab, 0, nmol * sizeof(float*), st);
   // kernel spectra and twiddles per group
   for (Group& g : b->groups) {
-    const size_t m = (size_t)g.n + 1;
-    std::vector<double> Gh(m * m * m);
-    if (!exx_host::kernel_spectrum_octant(g.n, g.h, kernel, 0.0, Gh.data())) {
+    exx_status_t gs = e == cudaSuccess ? group_tables(b, g, g.plane, &g.Gs, &g.tw, st) : EXX_ERR_CUDA;
+    if (gs != EXX_OK) {
       batch_free(b);
       delete b;
-      return EXX_ERR_INVALID_ARG;
+      return gs;
     }
-    const double L = 2.0 * g.n, scale = 1.0 / (L * L * L);
-    std::vector<double> gx(m), gy(2 * (size_t)g.n), gz(2 * (size_t)g.n);
-    g.ops->gains(gx.data(), gy.data(), gz.data());
-    std::vector<unsigned char> gf(exx::kernel_table_bytes(g.n, g.n, sizeof(float), g.ops->table_fold_y));
-    exx::build_kernel_table<float>(g.n, g.n, g.ops->table_fold_y, Gh.data(), scale, gx.data(),
-                                   gy.data(), gz.data(), gf.data());
-    std::vector<float> tw(2 * exx::twiddle_count(g.n));
-    exx::build_twiddles(g.n, tw.data());
-    if (!balloc(b, &g.Gs, gf.size()) || !balloc(b, &g.tw, tw.size() * sizeof(float))) {
-      batch_free(b);
-      delete b;
-      return EXX_ERR_OOM;
-    }
-    up(g.Gs, gf.data(), gf.size());
-    up(g.tw, tw.data(), tw.size() * sizeof(float));
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // host buffers die at scope end
-    if (e == cudaSuccess && g.ops->stage_table && !exx::make_ktab_map(&g.gmap, g.Gs, g.n, g.n))
-      e = cudaErrorInvalidValue;
-    if (e == cudaSuccess) e = g.ops->setup();
+    if (g.ops->stage_table && !g.plane && !exx::make_ktab_map(&g.gmap, g.Gs, g.n, g.n)) e = cudaErrorInvalidValue;
+    if (e == cudaSuccess) e = g.plane ? g.ops->plane_setup() : g.ops->setup();
   }
   if (!balloc(b, &b->d_err, 2 * sizeof(int))) {
     batch_free(b);
@@ -720,7 +748,36 @@ exx_status_t exx_batch_set_persistent(exx_batch_t b, int enable, void* cuda_stre
         mx = std::max(mx, std::max(g.nseg[0], g.nseg[1]));
       }
     if (segs.empty()) return EXX_OK;  // no group has a persistent kernel
-    // the queue reuses two workspace slots (those of the two pipeline lanes)
+    // the queue runs the slab pipeline on two workspace slots (those of the two
+    // pipeline lanes): its tables, and spectra padded along y
+    size_t xq = b->x_bytes;
+    for (Group& g : b->groups)
+      if (g.ops->persist_ok) {
+        if (g.plane && g.Gs_q == nullptr) {
+          const exx_status_t s = group_tables(b, g, false, &g.Gs_q, &g.tw_q, st);
+          if (s != EXX_OK) return s;
+        }
+        xq = std::max(xq, 2 * g.one);
+      }
+    if (xq > b->x_bytes) {
+      if (cudaStreamSynchronize(st) != cudaSuccess) return EXX_ERR_CUDA;
+      void *x1 = nullptr, *x2 = nullptr;
+      const size_t ws = b->ws;
+      if (!balloc(b, &x1, xq) || (b->X_2 && !balloc(b, &x2, xq))) {
+        if (x1) cudaFree(x1);
+        b->ws = ws;
+        return EXX_ERR_OOM;
+      }
+      cudaFree(b->X);
+      b->X = x1;
+      b->ws -= b->x_bytes;
+      if (b->X_2) {
+        cudaFree(b->X_2);
+        b->X_2 = x2;
+        b->ws -= b->x_bytes;
+      }
+      b->x_bytes = xq;
+    }
     if (b->X_2 == nullptr) {
       if (!balloc(b, &b->epart2, b->ep_bytes) || !balloc(b, &b->X_2, b->x_bytes) ||
           !balloc(b, &b->V_2, b->v_bytes))

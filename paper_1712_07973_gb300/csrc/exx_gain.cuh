@@ -47,11 +47,12 @@ template <> struct creal<F32c2> { using type = F32c; };
 // (F32c; a type with the same interface that does not round gives |d|^2 = 1).
 // L1O: the line split of the modelled pass (0: split_l1, the y pass; the z
 // pass of zconv uses split_z).
-template <int N, bool PER = false, typename S = F32c, int L1O = 0> struct GainModel {
+// X1O: the first factor of the modelled x split (0: split_x, the slab kernels).
+template <int N, bool PER = false, typename S = F32c, int L1O = 0, int X1O = 0> struct GainModel {
   using R = S;
   using C = typename cvec<S>::type;
   static constexpr int L = 2 * N, L1 = L1O ? L1O : split_l1(L), L2 = L / L1, H1 = L1 / 2;
-  static constexpr int X1 = split_x(N), X2 = N / X1;
+  static constexpr int X1 = X1O ? X1O : split_x(N), X2 = N / X1;
   static constexpr int G = PER ? L : N;  // input samples per line
   static constexpr int NIN = PER ? L1 : H1;
   static constexpr bool PX = !PER && (N % 2) == 0;

@@ -5,13 +5,16 @@
 
 #include <cmath>
 #include <cstddef>
+#include <vector>
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include "exx.h"
 #include "exx_gain.cuh"
 #include "exx_kernels.cuh"
 #include "exx_persist.cuh"
+#include "exx_plane.cuh"
 
 namespace exx {
 
@@ -42,6 +45,20 @@ struct Ops {
   void (*zconv)(void* X, const void* Gs, const void* tw, const CUtensorMap* gmap, double* epart,
                 int* err, int npair, bool energy_only, cudaStream_t st) = nullptr;
   bool stage_table = false;
+  // plane pipeline (exx_plane.cuh), where it is built: its own spectrum layout,
+  // kernel table and twiddles.  plane_ry = 2: needs a second spectrum buffer
+  bool plane_ok = false;
+  int plane_ry = 1;
+  int plane_ne = 1;  // energy partials per plane
+  cudaError_t (*plane_setup)() = nullptr;
+  void (*plane_gains)(double* gx, double* gy, double* gz) = nullptr;
+  size_t plane_twiddles = 0;  // complex values
+  void (*plane_build_twiddles)(void* out) = nullptr;
+  void (*xfwd)(const void* psi, const void* const* psi_tab, const int4* pairs, int npair, void* X, const void* tw,
+               long long n3, cudaStream_t st) = nullptr;
+  void (*plane)(const void* X, void* Y, const void* Gs, const void* tw, double* epart, int npair, bool energy_only,
+                cudaStream_t st) = nullptr;
+  void (*xinv)(const void* X, void* V, const void* tw, int npair, cudaStream_t st) = nullptr;
   void (*inv_yx)(const void* X3, void* V, const void* tw, int npair, cudaStream_t st) = nullptr;
   // persistent batched kernel (FP32, free boundary conditions, slab kernels
   // without clusters): threads per CTA, and the launch of a queue
@@ -217,6 +234,43 @@ void build_kernel_table(int n, int nz, bool fold_y, const double* octant, double
   }
 }
 
+// Twiddles of one line of the plane kernel: TA, TB (exx_plane.cuh).
+template <typename R, typename Ln> void build_line_twiddles(R*& out) {
+  auto put = [&](long e) {
+    const double a = -2.0 * M_PI * (double)(e % Ln::L) / (double)Ln::L;
+    *out++ = (R)std::cos(a);
+    *out++ = (R)std::sin(a);
+  };
+  for (int s = 0; s < (Ln::PER ? 1 : 2); ++s)
+    for (int n2 = 0; n2 < Ln::L2; ++n2)
+      for (int k1 = 0; k1 < Ln::H1; ++k1) put((long)n2 * (Ln::PER ? k1 : 2 * k1 + s));
+  for (int k1 = 0; k1 < Ln::L1; ++k1)
+    for (int m2 = 0; m2 < Ln::L2; ++m2) put((long)k1 * m2);
+}
+
+// Kernel table of the plane kernel: Gt[kx][kz][ky] as build_kernel_table's
+// unfolded one; ry = 2: the even ky, then the odd ky.
+template <typename R>
+void build_plane_table(int n, int nz, int ry, const double* octant, double scale, const double* gx, const double* gy,
+                       const double* gz, unsigned char* out) {
+  const long m = n + 1, L = 2 * n, LZ = 2 * nz;
+  R* G = reinterpret_cast<R*>(out);
+  std::vector<double> cy(L);
+  for (long k = 0; k < L; ++k) cy[k] = gy ? 1.0 / gy[k] : 1.0;
+#pragma omp parallel for schedule(static)
+  for (long kz = 0; kz < LZ; ++kz) {
+    const long kzf = kz <= nz ? kz : LZ - kz;
+    for (long kx = 0; kx < m; ++kx) {
+      const double c = scale / ((gx ? gx[kx] : 1.0) * (gz ? gz[kz] : 1.0));
+      R* row = G + (kx * LZ + kz) * L;
+      for (long ky = 0; ky < L; ++ky) {
+        const long kyf = ky <= n ? ky : L - ky;
+        row[ry == 2 ? (ky & 1) * n + (ky >> 1) : ky] = (R)(c * cy[ky] * octant[(kzf * m + kyf) * m + kx]);
+      }
+    }
+  }
+}
+
 // (N, PER): the x and y transforms; (NZ, PERZ): the z transform (mixed
 // boundary conditions: slab = periodic x, y with free z; wire = the reverse).
 template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> struct OpsImpl {
@@ -286,6 +340,7 @@ template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> stru
                                 : CTAS_B >= 2 ? 2 : 1;
   // ky-folded kernel table where the unfolded one would exceed 24 MB
   static constexpr bool fold_y = !mixed && !stage_g && (size_t)(N + 1) * (2 * N) * (2 * N) * sizeof(R) > (24u << 20);
+  static constexpr bool plane_ok = PlaneBuilt<R, G, PER, PERZ>::value && XCfg<R, N, PER>::ok && G >= 16;
   static constexpr bool ok = L1 != 0 && LZ1 != 0 && X1 != 0 && SA.fits && SC.fits && smem_b <= kSmemPerCTA;
   template <bool EO> static constexpr auto zk() {
     return &k_zconv<R, N, NW, MINB_B, stage_g, fold_y, PER, EO, NZ, PERZ>;
@@ -296,6 +351,11 @@ template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> stru
                                      QC == 0 && CL_A == 1 && CL_C == 1 && NT_A == NT_C;
   static constexpr int NT_P = NT_A;
   static constexpr int MINB_P = MINB_A < MINB_C ? MINB_A : MINB_C;
+  // slab pipeline: where the plane pipeline is not built (its kernels below are
+  // instantiated there only); its energy path also serves the allocation-free
+  // entry point, and the persistent kernel runs its per-CTA code
+  static constexpr bool slab_path = ok && !plane_ok;
+  static constexpr bool slab_energy = slab_path || (ok && sizeof(R) == 4 && !PER && !mixed && N <= EXX_NOALLOC_MAX_N);
   static constexpr size_t smem_p = smem_a > smem_c ? (smem_a > smem_b0 ? smem_a : smem_b0)
                                                    : (smem_c > smem_b0 ? smem_c : smem_b0);
   static constexpr auto pk() { return &k_persist<N, NT_P, MINB_P, fold_y>; }
@@ -319,6 +379,83 @@ template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> stru
     return cudaErrorNotSupported;
   }
 
+  // plane pipeline: every grid of 16 points and more whose spectrum plane, or
+  // half of it, fits an SM (FP32 up to 160^3 free and 128^3 periodic, FP64 up to
+  // 112^3 and 96^3).  Against the slab pipeline per call (FP32, two lanes): 96^3
+  // 32 orbitals 9.98 -> 8.50 ms, 160^3 32 orbitals 60.6 -> 46.6, 64^3 16 orbitals
+  // 0.782 -> 0.673, periodic 96^3 32 orbitals 3.96 -> 3.63; 16^3 4 orbitals 41.1 ->
+  // 41.0 us (launches either way; smaller grids stay on the slab pipeline)
+  static constexpr PlaneShape PS = plane_shape<R, G, PER, PERZ>();
+  static constexpr int RY = PS.ry;
+  using PC = PlaneCfg<R, G, PER, PERZ, RY, PS.nt, PS.minb, PS.ng>;
+  using XC = XCfg<R, N, PER>;
+  using YLn = PLine<G, PER>;
+  using ZLn = PLine<G, PERZ>;
+  static void plane_gains(double* gx, double* gy, double* gz) {
+    if constexpr (plane_ok) {
+      GainModel<N, PER, F32c, YLn::L1, XC::X1>::gains(gx, gy);
+      if constexpr (PC::SAME) {
+        for (int k = 0; k < L; ++k) gz[k] = gy[k];
+      } else {
+        std::vector<double> tx(NZ + 1);
+        GainModel<NZ, PERZ, F32c, ZLn::L1>::gains(tx.data(), gz);
+      }
+    }
+  }
+  static constexpr int plane_ne = PC::NE;
+  static constexpr size_t plane_ntw = 3 * (size_t)N + PC::TWN;
+  static void plane_build_twiddles(void* out) {
+    if constexpr (plane_ok) {
+      R* o = static_cast<R*>(out);
+      auto put = [&](long e) {
+        const double a = -M_PI * (double)(e % (2 * N)) / (double)N;
+        *o++ = (R)std::cos(a);
+        *o++ = (R)std::sin(a);
+      };
+      for (int k = 0; k < 2 * N; ++k) put(k);  // w^k
+      for (int k1 = 0; k1 < XC::X1; ++k1)      // TX
+        for (int n2 = 0; n2 < XC::X2; ++n2) put(2L * n2 * k1);
+      build_line_twiddles<R, YLn>(o);
+      if constexpr (!PC::SAME) build_line_twiddles<R, ZLn>(o);
+    }
+  }
+  template <bool EO> static constexpr auto plk() { return &k_plane<R, G, PER, PERZ, RY, PS.nt, PS.minb, PS.ng, EO>; }
+  static cudaError_t plane_setup() {
+    if constexpr (plane_ok) {
+      cudaError_t e = cudaFuncSetAttribute(plk<false>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PC::smem);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(plk<true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PC::smem);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_xfwd<R, N, PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)XC::smem);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_xinv<R, N, PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)XC::smem);
+      return e;
+    }
+    return cudaErrorNotSupported;
+  }
+  static void xfwd(const void* psi, const void* const* psi_tab, const int4* pairs, int npair, void* X, const void* tw,
+                   long long n3, cudaStream_t st) {
+    if constexpr (plane_ok)
+      k_xfwd<R, N, PER><<<dim3(npair, G * XC::NZB), XC::NT, XC::smem, st>>>(
+          static_cast<const R*>(psi), reinterpret_cast<const R* const*>(psi_tab), pairs, static_cast<C*>(X),
+          static_cast<const C*>(tw), n3);
+  }
+  static void plane(const void* X, void* Y, const void* Gs, const void* tw, double* epart, int npair, bool energy_only,
+                    cudaStream_t st) {
+    if constexpr (plane_ok) {
+      const int planes = npair * (N + 1), full = 152 * PC::MINB;
+      const int grid = planes < full ? planes : full;
+      auto k = energy_only ? plk<true>() : plk<false>();
+      k<<<grid, PC::NT, PC::smem, st>>>(static_cast<const C*>(X), static_cast<C*>(Y), static_cast<const R*>(Gs),
+                                        static_cast<const C*>(tw) + 3 * N, epart, npair, N + 1);
+    }
+  }
+  static void xinv(const void* X, void* V, const void* tw, int npair, cudaStream_t st) {
+    if constexpr (plane_ok)
+      k_xinv<R, N, PER><<<dim3(npair, G * XC::NZB), XC::NT, XC::smem, st>>>(
+          static_cast<const C*>(X), static_cast<R*>(V), static_cast<const C*>(tw));
+  }
+
   // gains of the x and y transforms, and of the z transform
   static void gains(double* gx, double* gy, double* gz) {
     GainModel<N, PER>::gains(gx, gy);
@@ -331,23 +468,25 @@ template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> stru
   }
 
   static cudaError_t setup() {
-    if constexpr (ok) {
-      cudaError_t e;
+    cudaError_t e = cudaErrorNotSupported;
+    if constexpr (slab_energy) {
       e = cudaFuncSetAttribute(k_fwd_xy<R, N, NT_A, MINB_A, QA, CL_A, PER>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_a);
-      if (e != cudaSuccess) return e;
-      e = cudaFuncSetAttribute(zk<false>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b);
-      if (e != cudaSuccess) return e;
-      e = cudaFuncSetAttribute(zk<true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b);
-      if (e != cudaSuccess) return e;
-      return cudaFuncSetAttribute(k_inv_yx<R, N, NT_C, MINB_C, QC, CL_C, PER>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(zk<true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b);
     }
-    return cudaErrorNotSupported;
+    if constexpr (slab_path) {
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(zk<false>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_inv_yx<R, N, NT_C, MINB_C, QC, CL_C, PER>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c);
+    }
+    return e;
   }
   static void fwd_xy(const void* psi, const void* const* psi_tab, const int4* pairs, int npair,
                      void* X, const void* tw, long long n3, cudaStream_t st) {
-    if constexpr (ok)
+    if constexpr (slab_energy)
       launch_slab<CL_A>(k_fwd_xy<R, N, NT_A, MINB_A, QA, CL_A, PER>, dim3(CL_A * npair, G), NT_A,
                         smem_a, st, static_cast<const R*>(psi),
                         reinterpret_cast<const R* const*>(psi_tab), pairs, static_cast<C*>(X),
@@ -355,20 +494,20 @@ template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> stru
   }
   static void zconv(void* X, const void* Gs, const void* tw, const CUtensorMap* gmap,
                     double* epart, int* err, int npair, bool energy_only, cudaStream_t st) {
-    if constexpr (ok) {
-      const dim3 grid(NYB, npair, N + 1);
-      CUtensorMap m{};
-      if (stage_g && gmap) m = *gmap;
+    const dim3 grid(NYB, npair, N + 1);
+    CUtensorMap m{};
+    if (stage_g && gmap) m = *gmap;
+    if constexpr (slab_energy)
       if (energy_only)
         zk<true>()<<<grid, 32 * NW, smem_b, st>>>(static_cast<C*>(X), static_cast<const R*>(Gs),
                                                   static_cast<const C*>(tw), epart, m, err);
-      else
+    if constexpr (slab_path)
+      if (!energy_only)
         zk<false>()<<<grid, 32 * NW, smem_b, st>>>(static_cast<C*>(X), static_cast<const R*>(Gs),
                                                    static_cast<const C*>(tw), epart, m, err);
-    }
   }
   static void inv_yx(const void* X, void* V, const void* tw, int npair, cudaStream_t st) {
-    if constexpr (ok)
+    if constexpr (slab_path)
       launch_slab<CL_C>(k_inv_yx<R, N, NT_C, MINB_C, QC, CL_C, PER>, dim3(G * CL_C, npair), NT_C,
                         smem_c, st, static_cast<const C*>(X), static_cast<R*>(V),
                         static_cast<const C*>(tw));
@@ -380,7 +519,7 @@ template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> stru
     o.grid = G;
     o.periodic = PER;
     o.periodic_z = PERZ;
-    o.supported = ok;
+    o.supported = ok || plane_ok;
     o.nyb = NYB;
     o.nt_a = NT_A;
     o.nt_c = NT_C;
@@ -399,6 +538,18 @@ template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> stru
     o.persist_ok = persist_ok;
     o.persist_nt = NT_P;
     if constexpr (persist_ok) o.persist = &persist;
+    o.plane_ok = plane_ok;
+    if constexpr (plane_ok) {
+      o.plane_ry = RY;
+      o.plane_ne = plane_ne;
+      o.plane_setup = &plane_setup;
+      if constexpr (sizeof(R) == 4) o.plane_gains = &plane_gains;
+      o.plane_twiddles = plane_ntw;
+      o.plane_build_twiddles = &plane_build_twiddles;
+      o.xfwd = &xfwd;
+      o.plane = &plane;
+      o.xinv = &xinv;
+    }
     return o;
   }
 };
