@@ -764,7 +764,7 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
       if (nl > 1 && used[l]) EXX_CUDA(p, cudaStreamWaitEvent(sl, p->ev_free[l], 0));
       {
         ProfScope ps(p, K_INV, sl);
-        if (p->plane) p->ops->xinv(Yt, Vt, p->tw, t.count, sl);
+        if (p->plane) p->ops->xinv(Yt, Vt, p->tw, t.count, 0, n, sl);
         else p->ops->inv_yx(X2, Vt, p->tw, t.count, sl);
       }
       if (nl > 1) {

@@ -355,7 +355,7 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
       if (apply) {
         if (nl > 1 && used[l] && cudaStreamWaitEvent(sl, b->ev_free[l], 0) != cudaSuccess)
           return EXX_ERR_CUDA;
-        if (g.plane) g.ops->xinv(Yl, Vl[l], g.tw, w.npair, sl);
+        if (g.plane) g.ops->xinv(Yl, Vl[l], g.tw, w.npair, 0, g.n, sl);
         else g.ops->inv_yx(Xl[l], Vl[l], g.tw, w.npair, sl);
         if (nl > 1 && (cudaEventRecord(b->ev_done[l], sl) != cudaSuccess ||
                        cudaStreamWaitEvent(st, b->ev_done[l], 0) != cudaSuccess))

@@ -563,32 +563,43 @@ __host__ __device__ constexpr int plane_x1(int N) {
     if (N % a == 0 && a * a >= N && smooth7(a) && smooth7(N / a)) return a;
   return 0;
 }
-// z-lines per CTA: the largest divisor of the grid up to 32, so that the
-// accesses to X[kx][y][z] are runs of up to 256 bytes and no CTA is partial
+// z-lines per CTA: 32 where that divides the grid (X[kx][y][z] in runs of 256
+// bytes), else its largest divisor up to 16, so that no CTA is partial (160^3:
+// 9.0 and 8.1 us per pair forward and inverse with 32, 9.9 and 12.0 with 16)
 __host__ __device__ constexpr int plane_zb(int G) {
-  for (int b = 32; b > 1; --b)
+  if (G % 32 == 0) return 32;
+  for (int b = 16; b > 1; --b)
     if (G % b == 0) return b;
   return 1;
 }
 // One CTA per (pair, y, block of ZB lines).  The transform takes two passes
-// and one exchange through S (row r of ZB lines at srow(r)).  On the spectrum
-// side a thread holds the two sub-DFTs q and X1 - q (q = 0: 0 and X1 / 2) of a
-// line: the frequencies k and N - k that the split into the Hermitian half
-// spectrum (and its inverse) combines are both its own, so the spectrum goes
-// from registers to memory (from memory to registers) with no further pass.
+// and one exchange through S.  On the spectrum side a thread holds the two
+// sub-DFTs q and X1 - q (q = 0: 0 and X1 / 2) of a line: the frequencies k and
+// N - k that the split into the Hermitian half spectrum (and its inverse)
+// combines are both its own, so the spectrum goes from registers to memory
+// (from memory to registers) with no further pass.
+// Forward, the samples come in whole rows through T[zl][x] (pairs of samples,
+// odd pitch) and every pass keeps its lanes along zl: read straight from memory,
+// eight or ten lanes per row and orbital, they kept the load/store unit 80% busy
+// at 160^3 (11.3 -> 9.0 us per pair; 64^3 0.87 -> 0.75).  Inverse, the samples of
+// one orbital pair go straight from registers to memory (a stage and its
+// barrier cost more: 8.1 -> 8.9 us at 160^3), lanes along x.
 template <typename R, int N, bool PER> struct XCfg {
   static constexpr int G = PER ? 2 * N : N;
   static constexpr int ZB = plane_zb(G), NZB = G / ZB;
   static constexpr int X1 = plane_x1(N), X2 = X1 ? N / X1 : 1;
-  static constexpr int SP = ZB | 1;
-  static constexpr bool ok = X1 != 0 && X2 <= 16;
-  static constexpr int UA = X2 * ZB;         // units (line, n2) of the sample side
+  static constexpr int GC = G / 2, TP = GC | 1;  // sample pairs per line, pitch of T
+  static constexpr bool ok = X1 != 0 && X2 <= 16 && G % 2 == 0;
+  static constexpr int UA = X2 * ZB;         // units (n2, line) of the sample side
   static constexpr int UB = (X1 / 2) * ZB;   // units (q, line) of the spectrum side
   static constexpr int most = UA > UB ? UA : UB;
-  static constexpr int NT = most >= 256 ? 256 : (most + 31) / 32 * 32;
-  static constexpr int MINB = sizeof(R) == 8 ? 512 / NT : X2 > 12 ? 640 / NT : 768 / NT;
-  // twiddles w^k (k < 2N) and TX[k1][n2] = w^(2 n2 k1) (N), S
-  static constexpr size_t smem = (3 * (size_t)N + (size_t)N * SP + (X1 ? N / X1 : 0) + 1) * sizeof(cplx<R>);
+  static constexpr int NT = most >= 320 ? 320 : (most + 31) / 32 * 32;
+  static constexpr int MINB = (sizeof(R) == 8 ? 512 : 1024) / NT;
+  // forward: twiddles w^k (k < 2N) and TX[k1][n2] = w^(2 n2 k1) (N), T, S[row][zl]
+  static constexpr size_t smem_f = (3 * (size_t)N + (size_t)ZB * TP + (size_t)N * ZB) * sizeof(cplx<R>);
+  // inverse: w^k, S with row r at srow(r) (pitch SP, skewed every X1 rows)
+  static constexpr int SP = ZB | 1;
+  static constexpr size_t smem_i = (2 * (size_t)N + (size_t)N * SP + (X1 ? N / X1 : 0) + 1) * sizeof(cplx<R>);
 };
 
 template <typename R, int N, bool PER>
@@ -597,39 +608,64 @@ k_xfwd(const R* __restrict__ psi0, const R* const* __restrict__ psi_tab, const i
        cplx<R>* __restrict__ X, const cplx<R>* __restrict__ tw_g, long long n3) {
   using C = cplx<R>;
   using K = XCfg<R, N, PER>;
-  constexpr int G = K::G, ZB = K::ZB, X1 = K::X1, X2 = K::X2, SP = K::SP, NT = K::NT;
+  constexpr int G = K::G, ZB = K::ZB, X1 = K::X1, X2 = K::X2, NT = K::NT, GC = K::GC, TP = K::TP;
   constexpr int XIN = PER ? X1 : X1 / 2;  // nonzero inputs of the length-X1 DFTs
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* tx = tw + 2 * N;
-  C* S = tx + N;
+  C* T = tx + N;
+  C* S = T + ZB * TP;
   const int tid = threadIdx.x;
-  const int p = blockIdx.x, y = blockIdx.y / K::NZB, z0 = (blockIdx.y - y * K::NZB) * ZB;
+  const int p = blockIdx.x / K::NZB, y = blockIdx.y, z0 = (blockIdx.x - p * K::NZB) * ZB;
   const int4 pr = pairs[p];
   const R* psi = psi_tab ? psi_tab[pr.w] : psi0;
   const R* __restrict__ pi = psi + (long long)pr.x * n3 + (long long)z0 * G * G + y * G;
   const R* __restrict__ pj = psi + (long long)pr.y * n3 + (long long)z0 * G * G + y * G;
-  for (int t = tid; t < 3 * N; t += NT) tw[t] = tw_g[t];
-  __syncthreads();
-  // samples: units (zl, n2), n2 fastest; z[m] = rho[2m] + i rho[2m+1], m = X2 n1 + n2
-#pragma unroll 1
-  for (int u = tid; u < K::UA; u += NT) {
-    const int zl = u / X2, n2 = u - zl * X2;
-    const R* ri = pi + (long long)zl * G * G + 2 * n2;
-    const R* rj = pj + (long long)zl * G * G + 2 * n2;
-    C v[X1];
+  // rho[2m] + i rho[2m+1], whole rows; paired loads where the caller's orbitals
+  // are aligned for them
+  if ((reinterpret_cast<size_t>(psi) & (sizeof(C) - 1)) == 0) {
+    constexpr int NL = (ZB * GC + NT - 1) / NT;
+    C a[NL], b[NL];
 #pragma unroll
-    for (int n1 = 0; n1 < XIN; ++n1)
-      v[n1] = mkc<C>(ri[2 * X2 * n1] * rj[2 * X2 * n1], ri[2 * X2 * n1 + 1] * rj[2 * X2 * n1 + 1]);
-    if constexpr (PER) dft<X1, 1, -1>(v);
-    else dft_halfin<X1, -1>(v);
-    C* col = S + srow<SP, X1>(n2 * X1) + zl;
-    col[0] = v[0];
+    for (int i = 0; i < NL; ++i) {
+      const int t = tid + i * NT, zl = t / GC, c = t - zl * GC;
+      if (ZB * GC % NT == 0 || t < ZB * GC) {
+        a[i] = __ldg(reinterpret_cast<const C*>(pi + (long long)zl * G * G) + c);
+        b[i] = __ldg(reinterpret_cast<const C*>(pj + (long long)zl * G * G) + c);
+      }
+    }
+    for (int t = tid; t < 3 * N; t += NT) tw[t] = tw_g[t];
 #pragma unroll
-    for (int k1 = 1; k1 < X1; ++k1) col[k1 * SP] = cmul(v[k1], tx[k1 * X2 + n2]);
+    for (int i = 0; i < NL; ++i) {
+      const int t = tid + i * NT, zl = t / GC, c = t - zl * GC;
+      if (ZB * GC % NT == 0 || t < ZB * GC) T[zl * TP + c] = mkc<C>(a[i].x * b[i].x, a[i].y * b[i].y);
+    }
+  } else {
+    for (int t = tid; t < 3 * N; t += NT) tw[t] = tw_g[t];
+    for (int t = tid; t < ZB * GC; t += NT) {
+      const int zl = t / GC, c = t - zl * GC;
+      const R* ri = pi + (long long)zl * G * G + 2 * c;
+      const R* rj = pj + (long long)zl * G * G + 2 * c;
+      T[zl * TP + c] = mkc<C>(ri[0] * rj[0], ri[1] * rj[1]);
+    }
   }
   __syncthreads();
-  // spectrum: units (q, zl), zl fastest; Z[a + X1 k2], Z[b + X1 k2]
+  // sample side: units (n2, zl), zl fastest; m = X2 n1 + n2
+#pragma unroll 1
+  for (int u = tid; u < K::UA; u += NT) {
+    const int n2 = u / ZB, zl = u - n2 * ZB;
+    C v[X1];
+#pragma unroll
+    for (int n1 = 0; n1 < XIN; ++n1) v[n1] = T[zl * TP + X2 * n1 + n2];
+    if constexpr (PER) dft<X1, 1, -1>(v);
+    else dft_halfin<X1, -1>(v);
+    C* col = S + n2 * X1 * ZB + zl;
+    col[0] = v[0];
+#pragma unroll
+    for (int k1 = 1; k1 < X1; ++k1) col[k1 * ZB] = cmul(v[k1], tx[k1 * X2 + n2]);
+  }
+  __syncthreads();
+  // spectrum side: units (q, zl), zl fastest; Z[a + X1 k2], Z[b + X1 k2]
   C* Xo = X + ((long long)p * (N + 1) * G + y) * G + z0;
   constexpr int KS = G * G;  // stride of kx
 #pragma unroll 1
@@ -639,8 +675,8 @@ k_xfwd(const R* __restrict__ psi0, const R* const* __restrict__ psi_tab, const i
     C va[X2], vb[X2];
 #pragma unroll
     for (int n2 = 0; n2 < X2; ++n2) {
-      va[n2] = S[srow<SP, X1>(n2 * X1) + a * SP + zl];
-      vb[n2] = S[srow<SP, X1>(n2 * X1) + b * SP + zl];
+      va[n2] = S[(n2 * X1 + a) * ZB + zl];
+      vb[n2] = S[(n2 * X1 + b) * ZB + zl];
     }
     dft<X2, 1, -1>(va);
     dft<X2, 1, -1>(vb);
@@ -693,36 +729,46 @@ template <typename C> EXX_HD void fold_step(C xk, C xm, C w, C& zk, C& zm) {
   zm = mkc<C>(e.x + o.y, o.x - e.y);
 }
 
+// The lines y0 .. y0 + ny - 1 of every pair: V[p][z][y - y0][x].
 template <typename R, int N, bool PER>
 __global__ void __launch_bounds__(XCfg<R, N, PER>::NT, XCfg<R, N, PER>::MINB)
-k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restrict__ tw_g) {
+k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restrict__ tw_g, int y0, int ny) {
   using C = cplx<R>;
   using K = XCfg<R, N, PER>;
   constexpr int G = K::G, ZB = K::ZB, X1 = K::X1, X2 = K::X2, SP = K::SP, NT = K::NT;
   constexpr int XOUT = PER ? X1 : X1 / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
-  C* S = tw + 3 * N;
+  C* S = tw + 2 * N;
   const int tid = threadIdx.x;
-  const int p = blockIdx.x, y = blockIdx.y / K::NZB, z0 = (blockIdx.y - y * K::NZB) * ZB;
-  const C* Xi = X + ((long long)p * (N + 1) * G + y) * G + z0;
+  const int p = blockIdx.x / K::NZB, yl = blockIdx.y, z0 = (blockIdx.x - p * K::NZB) * ZB;
+  const C* Xi = X + ((long long)p * (N + 1) * G + y0 + yl) * G + z0;
   constexpr int KS = G * G;
+  // spectrum side: units (q, zl), zl fastest; the first unit's values are under
+  // way during the set-up
+  C va[X2], vb[X2];
+  R xn = R(0);
+  auto load = [&](int u) {
+    const int q = u / ZB, zl = u - q * ZB;
+    const int a = q, b = q == 0 ? X1 / 2 : X1 - q;
+    const C* in = Xi + zl;
+#pragma unroll
+    for (int k2 = 0; k2 < X2; ++k2) {
+      va[k2] = __ldcs(in + (long long)(a + X1 * k2) * KS);
+      vb[k2] = __ldcs(in + (long long)(b + X1 * k2) * KS);
+    }
+    if (q == 0) xn = __ldcs(&in[(long long)N * KS].x);
+  };
+  if (tid < K::UB) load(tid);
   for (int t = tid; t < 2 * N; t += NT) tw[t] = tw_g[t];
   __syncthreads();
-  // spectrum: units (q, zl), zl fastest
 #pragma unroll 1
   for (int u = tid; u < K::UB; u += NT) {
     const int q = u / ZB, zl = u - q * ZB;
     const int a = q, b = q == 0 ? X1 / 2 : X1 - q;
-    const C* in = Xi + zl;
-    C va[X2], vb[X2];
-#pragma unroll
-    for (int k2 = 0; k2 < X2; ++k2) {
-      va[k2] = in[(long long)(a + X1 * k2) * KS];
-      vb[k2] = in[(long long)(b + X1 * k2) * KS];
-    }
+    if (u != tid) load(u);
     if (q == 0) {
-      const R xn = in[(long long)N * KS].x, x0 = va[0].x;
+      const R x0 = va[0].x;
       va[0] = mkc<C>(x0 + xn, x0 - xn);
 #pragma unroll
       for (int k2 = 1; 2 * k2 <= X2; ++k2) {
@@ -748,8 +794,8 @@ k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restri
     }
   }
   __syncthreads();
-  // samples: units (zl, m2), m2 fastest (coalesced writes along x)
-  R* Vz = V + ((long long)p * G + z0) * G * G + y * G;
+  // sample side: units (zl, m2), m2 fastest
+  R* Vz = V + (((long long)p * G + z0) * ny + yl) * G;
 #pragma unroll 1
   for (int u = tid; u < K::UA; u += NT) {
     const int zl = u / X2, m2 = u - zl * X2;
@@ -758,7 +804,7 @@ k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restri
     for (int k1 = 0; k1 < X1; ++k1) v[k1] = S[srow<SP, X1>(m2 * X1) + k1 * SP + zl];
     if constexpr (PER) dft<X1, 1, 1>(v);
     else dft_halfout<X1, 1>(v);
-    C* row = reinterpret_cast<C*>(Vz + (long long)zl * G * G) + m2;
+    C* row = reinterpret_cast<C*>(Vz + (long long)zl * ny * G) + m2;
 #pragma unroll
     for (int m1 = 0; m1 < XOUT; ++m1) row[X2 * m1] = v[m1];
   }

@@ -26,7 +26,7 @@ def shapes(tmp_path_factory):
              '\\"nt\\": %d, \\"c\\": %d, \\"ng\\": %d, \\"smem\\": %zu, \\"tcols\\": %d, \\"g\\": %d, \\"rows\\": %d, '
              '\\"per_z\\": %d, \\"x_nt\\": %d, \\"x_c\\": %d, \\"x_smem\\": %zu, \\"zb\\": %d, \\"x1\\": %d}\\n", bc, n, '
              'prec, (int)T::plane_ok, T::RY, K::NT, K::MINB, K::NG, K::smem, K::tcols, T::G, K::ROWS, '
-             '(int)K::Z::PER, X::NT, X::MINB, X::smem, X::ZB, X::X1);',
+             '(int)K::Z::PER, X::NT, X::MINB, X::smem_f, X::ZB, X::X1);',
              "}", "int main() {"]
     for bc, n, args in _registry():
         for prec, R in (("fp32", "float"), ("fp64", "double")):
