@@ -378,30 +378,40 @@ int default_tile(int N, int requested) {
 // k_accum launch: vector width 2 when aligned, full-tile specialisations
 template <typename R, int VEC>
 void launch_accum_v(int mode, const R* psi, const R* V, double* acc, const double* occ,
-                    const Tile& t, double c, double gs, long long n3, cudaStream_t st) {
+                    const Tile& t, double c, double gs, long long n3, int touch, R* out, cudaStream_t st) {
   const int threads = 256;
   const unsigned blocks = (unsigned)((n3 / VEC + threads - 1) / threads);
-  if (mode == 1)
-    k_accum<R, 8, VEC, 1><<<blocks, threads, 0, st>>>(psi, V, acc, occ, t.i0, t.ti, t.j0, t.tj,
-                                                       t.diag, c, gs, n3);
-  else if (mode == 2)
-    k_accum<R, 8, VEC, 2><<<blocks, threads, 0, st>>>(psi, V, acc, occ, t.i0, t.ti, t.j0, t.tj,
-                                                       t.diag, c, gs, n3);
-  else
-    k_accum<R, 8, VEC, 0><<<blocks, threads, 0, st>>>(psi, V, acc, occ, t.i0, t.ti, t.j0, t.tj,
-                                                       t.diag, c, gs, n3);
+  auto go = [&](auto k) {
+    k<<<blocks, threads, 0, st>>>(psi, V, acc, occ, t.i0, t.ti, t.j0, t.tj, t.diag, c, gs, n3, touch, out);
+  };
+  auto by_mode = [&](auto T) {
+    constexpr int t = decltype(T)::value;
+    go(mode == 1 ? k_accum<R, 8, VEC, 1, t> : mode == 2 ? k_accum<R, 8, VEC, 2, t> : k_accum<R, 8, VEC, 0, t>);
+  };
+  if constexpr (VEC == 16 / (int)sizeof(R)) {
+    switch (touch) {
+      case 0: return by_mode(ic<0>{});
+      case T_FIRST_I: return by_mode(ic<T_FIRST_I>{});
+      case T_FIRST_J: return by_mode(ic<T_FIRST_J>{});
+      case T_LAST_I: return by_mode(ic<T_LAST_I>{});
+      case T_FIRST_I | T_LAST_I: return by_mode(ic<T_FIRST_I | T_LAST_I>{});
+      case T_FIRST_J | T_LAST_I: return by_mode(ic<T_FIRST_J | T_LAST_I>{});
+      default: break;
+    }
+  }
+  by_mode(ic<-1>{});
 }
 template <typename R>
 void launch_accum(bool v2, int mode, const R* psi, const R* V, double* acc, const double* occ,
-                  const Tile& t, double c, double gs, long long n3, cudaStream_t st) {
+                  const Tile& t, double c, double gs, long long n3, int touch, R* out, cudaStream_t st) {
   if constexpr (sizeof(R) == 4) {  // four FP32 values per thread: -4% at 160^3
     if (v2 && (n3 % 4) == 0) {
-      launch_accum_v<R, 4>(mode, psi, V, acc, occ, t, c, gs, n3, st);
+      launch_accum_v<R, 4>(mode, psi, V, acc, occ, t, c, gs, n3, touch, out, st);
       return;
     }
   }
-  if (v2) launch_accum_v<R, 2>(mode, psi, V, acc, occ, t, c, gs, n3, st);
-  else launch_accum_v<R, 1>(mode, psi, V, acc, occ, t, c, gs, n3, st);
+  if (v2) launch_accum_v<R, 2>(mode, psi, V, acc, occ, t, c, gs, n3, touch, out, st);
+  else launch_accum_v<R, 1>(mode, psi, V, acc, occ, t, c, gs, n3, touch, out, st);
 }
 
 extern "C" {
@@ -672,7 +682,7 @@ exx_status_t exx_plan_info(exx_plan_t p, int* tile, int* ntiles, size_t* workspa
   if (tile) *tile = p->T;
   if (ntiles) *ntiles = nt;
   if (workspace_bytes) *workspace_bytes = p->ws;
-  const bool conv = p->vacc != nullptr;
+  const bool conv = p->vacc != nullptr && p->sharded;  // else part of the accumulation
   if (launches_apply) *launches_apply = 5 * nt + 1 + (conv ? 1 : 0);
   if (launches_energy) *launches_energy = 3 * nt + 1;
   return EXX_OK;
@@ -700,8 +710,10 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
   const int nper = p->nper;
   double* acc = nullptr;
   if (apply) {
+    // every orbital's first update clears and (FP32 output) its last converts,
+    // where this plan runs all tiles; a shard's tiles need not hold either
     acc = p->vacc ? p->vacc : static_cast<double*>(vxpsi);
-    EXX_CUDA(p, cudaMemsetAsync(acc, 0, (size_t)N * n3 * sizeof(double), st));
+    if (p->sharded) EXX_CUDA(p, cudaMemsetAsync(acc, 0, (size_t)N * n3 * sizeof(double), st));
   }
   const double c = -p->alpha;
   const double gs = grad ? 2.0 * h3 : 0.0;
@@ -761,10 +773,23 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
                                                                   p->Epair);
     }
     if (apply) {
+      // vector width: 4 (FP32) or 2 values per thread when n^3 and the
+      // caller's pointers allow aligned vector accesses
+      const bool row_end = ti + 1 == p->tiles.size() || p->tiles[ti + 1].i0 != t.i0;
+      int touch = 0;
+      if (!p->sharded) {
+        if (t.i0 == 0) touch = t.diag ? T_FIRST_I : T_FIRST_J;
+        if (row_end && p->vacc) touch |= T_LAST_I;  // (no conversion of an FP64 output)
+      }
+      float* out = (touch & T_LAST_I) ? static_cast<float*>(vxpsi) : nullptr;
+      const bool al = ((uintptr_t)psi % 16 == 0) && ((uintptr_t)acc % 16 == 0) &&
+                      (!p->vacc || (uintptr_t)vxpsi % 16 == 0);
+      const bool v2 = al && (n3 % 2) == 0;
+      const int mode = (t.ti == 8 && t.tj == 8) ? (t.diag ? 2 : 1) : 0;
       if (nl > 1 && used[l]) EXX_CUDA(p, cudaStreamWaitEvent(sl, p->ev_free[l], 0));
       {
         ProfScope ps(p, K_INV, sl);
-        if (p->plane) p->ops->xinv(Yt, Vt, p->tw, t.count, 0, n, sl);
+        if (p->plane) p->ops->xinv(Yt, Vt, p->tw, t.count, sl);
         else p->ops->inv_yx(X2, Vt, p->tw, t.count, sl);
       }
       if (nl > 1) {
@@ -772,31 +797,17 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
         EXX_CUDA(p, cudaStreamWaitEvent(st, p->ev_done[l], 0));
       }
       used[l] = true;
-      ProfScope ps(p, K_ACCUM, st);
-      // vector width: 4 (FP32) or 2 values per thread when n^3 and the
-      // caller's pointers allow aligned vector accesses
-      const bool al = ((uintptr_t)psi % 16 == 0) && ((uintptr_t)acc % 16 == 0);
-      const bool v2 = al && (n3 % 2) == 0;
-      const int mode = (t.ti == 8 && t.tj == 8) ? (t.diag ? 2 : 1) : 0;
-      if (p->prec == EXX_FP64)
-        launch_accum<double>(v2, mode, static_cast<const double*>(psi),
-                             static_cast<const double*>(Vt), acc, p->d_occ, t, c, gs, n3, st);
-      else
-        launch_accum<float>(v2, mode, static_cast<const float*>(psi),
-                            static_cast<const float*>(Vt), acc, p->d_occ, t, c, gs, n3, st);
-      if (nl > 1) EXX_CUDA(p, cudaEventRecord(p->ev_free[l], st));
-    }
-    const bool row_end = ti + 1 == p->tiles.size() || p->tiles[ti + 1].i0 != t.i0;
-    if (ov && apply && row_end) {
-      const int b = t.i0 / p->T;
-      if (p->vacc) {
-        ProfScope ps(p, K_CONV, st);
-        const long long cnt = (long long)t.ti * n3, off = (long long)t.i0 * n3;
-        long long blocks = (cnt + 255) / 256;
-        if (blocks > 152 * 32) blocks = 152 * 32;
-        k_to_float<<<(int)blocks, 256, 0, st>>>(p->vacc + off, static_cast<float*>(vxpsi) + off, cnt);
+      {
+        ProfScope ps(p, K_ACCUM, st);
+        if (p->prec == EXX_FP64)
+          launch_accum<double>(v2, mode, static_cast<const double*>(psi), static_cast<const double*>(Vt), acc,
+                               p->d_occ, t, c, gs, n3, touch, nullptr, st);
+        else
+          launch_accum<float>(v2, mode, static_cast<const float*>(psi), static_cast<const float*>(Vt), acc,
+                              p->d_occ, t, c, gs, n3, touch, out, st);
       }
-      EXX_CUDA(p, cudaEventRecord((*ov->out)[b], st));
+      if (nl > 1) EXX_CUDA(p, cudaEventRecord(p->ev_free[l], st));
+      if (ov && row_end) EXX_CUDA(p, cudaEventRecord((*ov->out)[t.i0 / p->T], st));
     }
   }
   if (nl > 1)  // join: every lane's pair energies (and, for apply, V reads) are done
@@ -808,7 +819,7 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
     ProfScope ps(p, K_TOTAL, st);
     k_exx_total<<<1, 256, 0, st>>>(p->Epair, p->P, N, p->d_occ, p->alpha, E_dev ? E_dev : p->E_dev);
   }
-  if (apply && p->vacc && !ov) {
+  if (apply && p->vacc && p->sharded) {
     ProfScope ps(p, K_CONV, st);
     const long long tot = (long long)N * n3;
     long long blocks = (tot + 255) / 256;

@@ -280,7 +280,9 @@ void build_segments(exx_batch_t b, Group& g, bool apply, bool stall, std::vector
 }
 
 exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaStream_t st) {
-  if (apply) {
+  // launch per pass: every orbital's first update clears and its last converts
+  // (TileDesc::touch); the persistent queue clears and converts in passes
+  if (apply && b->persistent) {
     long long tot = 0;
     for (const Mol& m : b->mol) tot += (long long)m.N * m.n * m.n * m.n;
     if (cudaMemsetAsync(b->vacc, 0, (size_t)tot * sizeof(double), st) != cudaSuccess) return EXX_ERR_CUDA;
@@ -355,22 +357,23 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
       if (apply) {
         if (nl > 1 && used[l] && cudaStreamWaitEvent(sl, b->ev_free[l], 0) != cudaSuccess)
           return EXX_ERR_CUDA;
-        if (g.plane) g.ops->xinv(Yl, Vl[l], g.tw, w.npair, 0, g.n, sl);
+        if (g.plane) g.ops->xinv(Yl, Vl[l], g.tw, w.npair, sl);
         else g.ops->inv_yx(Xl[l], Vl[l], g.tw, w.npair, sl);
         if (nl > 1 && (cudaEventRecord(b->ev_done[l], sl) != cudaSuccess ||
                        cudaStreamWaitEvent(st, b->ev_done[l], 0) != cudaSuccess))
           return EXX_ERR_CUDA;
         used[l] = true;
+        float* const* out = b->persistent ? nullptr : b->d_vx_tab;
         const bool v2 = b->vec2 && (n3 % 2) == 0;
         const int threads = 256;
         const long long blocks = (n3 / (v2 ? 2 : 1) + threads - 1) / threads;
         if (v2)
           k_accum_batch<float, 8, 2><<<dim3((unsigned)blocks, w.ntile), threads, 0, st>>>(
-              b->d_psi_tab, static_cast<const float*>(Vl[l]), b->d_vacc_tab, b->d_occ,
+              b->d_psi_tab, static_cast<const float*>(Vl[l]), b->d_vacc_tab, out, b->d_occ,
               b->d_tiles + w.tile_off, grad ? 1 : 0, n3);
         else
           k_accum_batch<float, 8, 1><<<dim3((unsigned)blocks, w.ntile), threads, 0, st>>>(
-              b->d_psi_tab, static_cast<const float*>(Vl[l]), b->d_vacc_tab, b->d_occ,
+              b->d_psi_tab, static_cast<const float*>(Vl[l]), b->d_vacc_tab, out, b->d_occ,
               b->d_tiles + w.tile_off, grad ? 1 : 0, n3);
         if (nl > 1 && cudaEventRecord(b->ev_free[l], st) != cudaSuccess) return EXX_ERR_CUDA;
       }
@@ -382,7 +385,7 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
           cudaStreamWaitEvent(st, b->ev_done[l], 0) != cudaSuccess)
         return EXX_ERR_CUDA;
   k_exx_total_batch<<<b->nmol, 256, 0, st>>>(b->Epair, b->d_mt, b->d_occ, E_dev);
-  if (apply && b->have_vx) {
+  if (apply && b->have_vx && b->persistent) {
     long long mx = 0;
     for (const Mol& m : b->mol) mx = std::max(mx, (long long)m.N * m.n * m.n * m.n);
     const long long blocks = std::min<long long>((mx + 255) / 256, 1024);
@@ -544,6 +547,7 @@ exx_status_t exx_batch_create(exx_batch_t* out, int nmol, const exx_mol_desc* mo
           t.c = -m.alpha;
           t.g2h3 = 2.0 * m.h * m.h * m.h;
           t.voff = 0;
+          t.touch = (bi == 0 ? (t.diag ? T_FIRST_I : T_FIRST_J) : 0) | (bj == nb - 1 ? T_LAST_I : 0);
           std::vector<int4> ps;
           for (int a = 0; a < t.ti; ++a)
             for (int c = t.diag ? a : 0; c < t.tj; ++c) {
@@ -841,7 +845,7 @@ exx_status_t exx_batch_info(exx_batch_t b, int* ngroups, int* nwaves, size_t* wo
   if (nwaves) *nwaves = nw;
   if (workspace_bytes) *workspace_bytes = b->ws;
   if (launches_apply) {
-    int la = 2;  // E_x totals and the conversion of the outputs
+    int la = b->persistent ? 2 : 1;  // E_x totals (and the conversion of the outputs)
     for (const Group& g : b->groups)
       la += (b->persistent && g.ops->persist_ok) ? 1 : 5 * (int)g.waves.size();
     *launches_apply = la;

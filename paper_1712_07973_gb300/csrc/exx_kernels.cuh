@@ -872,28 +872,45 @@ __device__ __forceinline__ void vload(const R* p, R (&v)[VEC]) {
     for (int e = 0; e < VEC; ++e) v[e] = q[e];
   }
 }
-// vx[0..VEC) += c * a  (FP64)
+// vx[0..VEC) += c * a  (FP64); first: the accumulator counts as zero and is
+// not read; out != null: the sum goes there in the working precision (the
+// orbital's last update), not back to the accumulator.  The same sums, bit for
+// bit, as clearing, adding and converting in passes of their own.
 template <typename R, int VEC, bool COH = false>
-__device__ __forceinline__ void vacc(double* p, double c, const R (&a)[VEC]) {
-  if constexpr (VEC == 4) {
-    double2* q = reinterpret_cast<double2*>(p);
-    double2 u = ldx<COH>(q), w = ldx<COH>(q + 1);
-    u.x += c * (double)a[0];
-    u.y += c * (double)a[1];
-    w.x += c * (double)a[2];
-    w.y += c * (double)a[3];
-    q[0] = u;
-    q[1] = w;
-  } else if constexpr (VEC == 2) {
-    double2* q = reinterpret_cast<double2*>(p);
-    double2 u = ldx<COH>(q);
-    u.x += c * (double)a[0];
-    u.y += c * (double)a[1];
-    q[0] = u;
+__device__ __forceinline__ void vacc(double* p, double c, const R (&a)[VEC], bool first, R* out) {
+  // (selects rather than branches: the loads stay ahead with the tile's others)
+  double u[VEC];
+  if constexpr (VEC == 1) {
+    u[0] = first ? 0.0 : ldx<COH>(p);
   } else {
-    p[0] = ldx<COH>(p) + c * (double)a[0];
+#pragma unroll
+    for (int e = 0; e < VEC; e += 2) {
+      double2 t = make_double2(0.0, 0.0);
+      if (!first) t = ldx<COH>(reinterpret_cast<const double2*>(p + e));
+      u[e] = t.x;
+      u[e + 1] = t.y;
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) u[e] += c * (double)a[e];
+  if (out != nullptr) {
+    if constexpr (sizeof(R) == 4 && VEC == 4) {
+      *reinterpret_cast<float4*>(out) = make_float4((float)u[0], (float)u[1], (float)u[2], (float)u[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) out[e] = (R)u[e];
+    }
+  } else if constexpr (VEC == 1) {
+    p[0] = u[0];
+  } else {
+#pragma unroll
+    for (int e = 0; e < VEC; e += 2) *reinterpret_cast<double2*>(p + e) = make_double2(u[e], u[e + 1]);
   }
 }
+
+// Which of a tile's updates are the first or the last of their orbitals in a
+// call (bits): 1 first of block I, 2 first of block J, 4 last of block I.
+enum Touch { T_FIRST_I = 1, T_FIRST_J = 2, T_LAST_I = 4 };
 
 // Products and accumulation of one tile at the VEC mesh points from r.
 // MODE 0: any tile; MODE 1: full off-diagonal tile (ti = tj = TM); MODE 2:
@@ -904,12 +921,13 @@ __device__ __forceinline__ void vacc(double* p, double c, const R (&a)[VEC]) {
 // gs = 0: the exchange action, vx_k += c * sum; gs > 0: the gradient of E_x,
 // vx_k += c gs f_k * sum (gs = 2 h^3: dE_x/dpsi_k = 2 f_k h^3 (Vx psi)_k,
 // Eq. daction), the per-orbital factor folded into the FP64 accumulation.
+// touch: Touch bits; out: the output that takes an orbital's last update.
 template <typename R, int TM, int VEC, int MODE, bool COH = false>
 __device__ __forceinline__ void accum_tile(const R* __restrict__ psi, const R* __restrict__ V,
                                            double* __restrict__ vx,
                                            const double* __restrict__ occ, int i0, int ti_,
                                            int j0, int tj_, int diag_, double c, double gs,
-                                           long long n3, long long r) {
+                                           long long n3, long long r, int touch, R* out) {
   const int ti = MODE ? TM : ti_, tj = MODE ? TM : tj_;
   const bool diag = MODE == 2 ? true : MODE == 1 ? false : diag_ != 0;
   R fi[TM];
@@ -953,25 +971,30 @@ __device__ __forceinline__ void accum_tile(const R* __restrict__ psi, const R* _
       for (int e = 0; e < VEC; ++e) ai[b][e] += aj[e];
     } else {
       const double cb = gs != 0.0 ? c * (gs * occ[j0 + b]) : c;
-      vacc<R, VEC, COH>(vx + (long long)(j0 + b) * n3 + r, cb, aj);
+      vacc<R, VEC, COH>(vx + (long long)(j0 + b) * n3 + r, cb, aj, (touch & T_FIRST_J) != 0, nullptr);
     }
   }
 #pragma unroll
   for (int a = 0; a < TM; ++a)
     if (a < ti) {
       const double ca = gs != 0.0 ? c * (gs * occ[i0 + a]) : c;
-      vacc<R, VEC, COH>(vx + (long long)(i0 + a) * n3 + r, ca, ai[a]);
+      const long long o = (long long)(i0 + a) * n3 + r;
+      vacc<R, VEC, COH>(vx + o, ca, ai[a], (touch & T_FIRST_I) != 0, out != nullptr ? out + o : nullptr);
     }
 }
 
-template <typename R, int TM, int VEC, int MODE>
+// TOUCH: the tile's Touch bits at compile time (a branch around an accumulator's
+// load keeps it from being issued ahead: 1.90 -> 2.16 us per pair at 96^3), or -1:
+// given by touch.
+template <typename R, int TM, int VEC, int MODE, int TOUCH>
 __global__ void __launch_bounds__(256, (sizeof(R) == 4 && MODE == 0) ? 3 : 2)
 k_accum(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__ vx,
         const double* __restrict__ occ, int i0, int ti, int j0, int tj, int diag, double c,
-        double gs, long long n3) {
+        double gs, long long n3, int touch, R* out) {
   const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * VEC;
   if (r >= n3) return;
-  accum_tile<R, TM, VEC, MODE>(psi, V, vx, occ, i0, ti, j0, tj, diag, c, gs, n3, r);
+  accum_tile<R, TM, VEC, MODE>(psi, V, vx, occ, i0, ti, j0, tj, diag, c, gs, n3, r,
+                               TOUCH < 0 ? touch : TOUCH, TOUCH < 0 || (TOUCH & T_LAST_I) ? out : nullptr);
 }
 
 // Tile descriptor of a batched wave (tiles of different molecules, or of
@@ -983,14 +1006,18 @@ struct TileDesc {
   int occ_off;
   double c;   // -alpha of the molecule
   double g2h3;  // 2 h^3 of the molecule (gradient calls)
+  int touch;    // Touch bits
 };
 
 // One tile per blockIdx.y; full tiles take the specialised bodies (the branch
 // is uniform over a block).  grad != 0: gradient of E_x (see accum_tile).
+// vx_out (table of output arrays): the tiles' Touch bits count; null: they do
+// not (the accumulators are cleared and converted in passes of their own).
 template <typename R, int TM, int VEC, bool COH>
 __device__ __forceinline__ void accum_batch_unit(const R* const* __restrict__ psi_tab,
                                                  const R* __restrict__ V,
                                                  double* const* __restrict__ vx_tab,
+                                                 R* const* __restrict__ vx_out,
                                                  const double* __restrict__ occ,
                                                  const TileDesc* __restrict__ tiles, int grad,
                                                  long long n3, const int bx, const int by,
@@ -1003,22 +1030,24 @@ __device__ __forceinline__ void accum_batch_unit(const R* const* __restrict__ ps
   const double* __restrict__ oc = occ + t.occ_off;
   const R* __restrict__ Vt = V + (long long)t.voff * n3;
   const double gs = grad ? t.g2h3 : 0.0;
+  const int touch = vx_out ? t.touch : 0;
+  R* out = (touch & T_LAST_I) ? vx_out[t.mol] : nullptr;
   if (t.ti == TM && t.tj == TM) {
     if (t.diag)
-      accum_tile<R, TM, VEC, 2, COH>(psi, Vt, vx, oc, t.i0, TM, t.j0, TM, 1, t.c, gs, n3, r);
+      accum_tile<R, TM, VEC, 2, COH>(psi, Vt, vx, oc, t.i0, TM, t.j0, TM, 1, t.c, gs, n3, r, touch, out);
     else
-      accum_tile<R, TM, VEC, 1, COH>(psi, Vt, vx, oc, t.i0, TM, t.j0, TM, 0, t.c, gs, n3, r);
+      accum_tile<R, TM, VEC, 1, COH>(psi, Vt, vx, oc, t.i0, TM, t.j0, TM, 0, t.c, gs, n3, r, touch, out);
   } else {
-    accum_tile<R, TM, VEC, 0, COH>(psi, Vt, vx, oc, t.i0, t.ti, t.j0, t.tj, t.diag, t.c, gs, n3, r);
+    accum_tile<R, TM, VEC, 0, COH>(psi, Vt, vx, oc, t.i0, t.ti, t.j0, t.tj, t.diag, t.c, gs, n3, r, touch, out);
   }
 }
 
 template <typename R, int TM, int VEC>
 __global__ void __launch_bounds__(256, 2)
 k_accum_batch(const R* const* __restrict__ psi_tab, const R* __restrict__ V,
-              double* const* __restrict__ vx_tab, const double* __restrict__ occ,
-              const TileDesc* __restrict__ tiles, int grad, long long n3) {
-  accum_batch_unit<R, TM, VEC, false>(psi_tab, V, vx_tab, occ, tiles, grad, n3, blockIdx.x,
+              double* const* __restrict__ vx_tab, R* const* __restrict__ vx_out,
+              const double* __restrict__ occ, const TileDesc* __restrict__ tiles, int grad, long long n3) {
+  accum_batch_unit<R, TM, VEC, false>(psi_tab, V, vx_tab, vx_out, occ, tiles, grad, n3, blockIdx.x,
                                       blockIdx.y, blockDim.x);
 }
 

@@ -58,7 +58,7 @@ struct Ops {
                long long n3, cudaStream_t st) = nullptr;
   void (*plane)(const void* X, void* Y, const void* Gs, const void* tw, double* epart, int npair, bool energy_only,
                 cudaStream_t st) = nullptr;
-  void (*xinv)(const void* X, void* V, const void* tw, int npair, int y0, int ny, cudaStream_t st) = nullptr;
+  void (*xinv)(const void* X, void* V, const void* tw, int npair, cudaStream_t st) = nullptr;
   void (*inv_yx)(const void* X3, void* V, const void* tw, int npair, cudaStream_t st) = nullptr;
   // persistent batched kernel (FP32, free boundary conditions, slab kernels
   // without clusters): threads per CTA, and the launch of a queue
@@ -450,10 +450,10 @@ template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> stru
                                         static_cast<const C*>(tw) + 3 * N, epart, npair, N + 1);
     }
   }
-  static void xinv(const void* X, void* V, const void* tw, int npair, int y0, int ny, cudaStream_t st) {
+  static void xinv(const void* X, void* V, const void* tw, int npair, cudaStream_t st) {
     if constexpr (plane_ok)
-      k_xinv<R, N, PER><<<dim3(npair * XC::NZB, ny), XC::NT, XC::smem_i, st>>>(
-          static_cast<const C*>(X), static_cast<R*>(V), static_cast<const C*>(tw), y0, ny);
+      k_xinv<R, N, PER><<<dim3(npair * XC::NZB, G), XC::NT, XC::smem_i, st>>>(
+          static_cast<const C*>(X), static_cast<R*>(V), static_cast<const C*>(tw));
   }
 
   // gains of the x and y transforms, and of the z transform

@@ -164,10 +164,10 @@ __global__ void __launch_bounds__(NT, MINB) k_persist(const PersistArgs a) {
       } else {
         const int t = u / a.nblk, b = u - t * a.nblk;
         if (a.vec2)
-          accum_batch_unit<float, 8, 2, true>(a.psi_tab, a.V[sg.slot], a.vx_tab, a.occ,
+          accum_batch_unit<float, 8, 2, true>(a.psi_tab, a.V[sg.slot], a.vx_tab, nullptr, a.occ,
                                               a.tiles + sg.tile_off, a.grad, a.n3, b, t, NT);
         else
-          accum_batch_unit<float, 8, 1, true>(a.psi_tab, a.V[sg.slot], a.vx_tab, a.occ,
+          accum_batch_unit<float, 8, 1, true>(a.psi_tab, a.V[sg.slot], a.vx_tab, nullptr, a.occ,
                                               a.tiles + sg.tile_off, a.grad, a.n3, b, t, NT);
       }
     }

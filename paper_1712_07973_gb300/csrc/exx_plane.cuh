@@ -729,10 +729,9 @@ template <typename C> EXX_HD void fold_step(C xk, C xm, C w, C& zk, C& zm) {
   zm = mkc<C>(e.x + o.y, o.x - e.y);
 }
 
-// The lines y0 .. y0 + ny - 1 of every pair: V[p][z][y - y0][x].
 template <typename R, int N, bool PER>
 __global__ void __launch_bounds__(XCfg<R, N, PER>::NT, XCfg<R, N, PER>::MINB)
-k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restrict__ tw_g, int y0, int ny) {
+k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restrict__ tw_g) {
   using C = cplx<R>;
   using K = XCfg<R, N, PER>;
   constexpr int G = K::G, ZB = K::ZB, X1 = K::X1, X2 = K::X2, SP = K::SP, NT = K::NT;
@@ -741,8 +740,8 @@ k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restri
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* S = tw + 2 * N;
   const int tid = threadIdx.x;
-  const int p = blockIdx.x / K::NZB, yl = blockIdx.y, z0 = (blockIdx.x - p * K::NZB) * ZB;
-  const C* Xi = X + ((long long)p * (N + 1) * G + y0 + yl) * G + z0;
+  const int p = blockIdx.x / K::NZB, y = blockIdx.y, z0 = (blockIdx.x - p * K::NZB) * ZB;
+  const C* Xi = X + ((long long)p * (N + 1) * G + y) * G + z0;
   constexpr int KS = G * G;
   // spectrum side: units (q, zl), zl fastest; the first unit's values are under
   // way during the set-up
@@ -795,7 +794,7 @@ k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restri
   }
   __syncthreads();
   // sample side: units (zl, m2), m2 fastest
-  R* Vz = V + (((long long)p * G + z0) * ny + yl) * G;
+  R* Vz = V + (((long long)p * G + z0) * G + y) * G;
 #pragma unroll 1
   for (int u = tid; u < K::UA; u += NT) {
     const int zl = u / X2, m2 = u - zl * X2;
@@ -804,7 +803,7 @@ k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restri
     for (int k1 = 0; k1 < X1; ++k1) v[k1] = S[srow<SP, X1>(m2 * X1) + k1 * SP + zl];
     if constexpr (PER) dft<X1, 1, 1>(v);
     else dft_halfout<X1, 1>(v);
-    C* row = reinterpret_cast<C*>(Vz + (long long)zl * ny * G) + m2;
+    C* row = reinterpret_cast<C*>(Vz + (long long)zl * G * G) + m2;
 #pragma unroll
     for (int m1 = 0; m1 < XOUT; ++m1) row[X2 * m1] = v[m1];
   }
