@@ -168,6 +168,40 @@ __global__ void k_exx_total(const double* __restrict__ Epair, long long P, int N
   if (threadIdx.x == 0) *E = -0.5 * alpha * red[0];
 }
 
+// Both for a call of a single tile (npair = P pairs): the warps take the pairs in
+// turn, then the first 256 threads sum as k_exx_total.
+__global__ void __launch_bounds__(1024) k_pair_energy_total(const double* __restrict__ epart, int nper,
+                                                            const int4* __restrict__ pairs, int npair, double h3,
+                                                            double* Epair, int N, const double* __restrict__ occ,
+                                                            double alpha, double* __restrict__ E) {
+  __shared__ double red[256];
+  const int lane = threadIdx.x & 31;
+  for (int w = threadIdx.x >> 5; w < npair; w += 32) {
+    double s = 0.0;
+    for (int t = lane; t < nper; t += 32) s += epart[(long long)w * nper + t];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) Epair[pairs[w].z] = h3 * s;
+  }
+  __syncthreads();
+  if (threadIdx.x < 256) {
+    double s = 0.0;
+    for (long long g = threadIdx.x; g < npair; g += 256) {
+      int i, j;
+      tri_decode(g, N, &i, &j);
+      const double m = (i == j) ? 1.0 : 2.0;
+      s += m * occ[i] * occ[j] * Epair[g];
+    }
+    red[threadIdx.x] = s;
+  }
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) *E = -0.5 * alpha * red[0];
+}
+
 __global__ void k_to_float(const double* __restrict__ a, float* __restrict__ b, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
@@ -375,12 +409,22 @@ int default_tile(int N, int requested) {
 
 }  // namespace
 
+// Below this many CTAs of points (152 SMs) one orbital per CTA row: 24^3 5 orbitals
+// 16 -> 6 us, 48^3 0.46 -> 0.41 us per pair, 56^3 (172 CTAs) 0.88 -> 0.70; 64^3 (256
+// CTAs) 0.71 -> 0.77, its potentials read twice.
+constexpr unsigned kWideBlocks = 200;
 // k_accum launch: vector width 2 when aligned, full-tile specialisations
 template <typename R, int VEC>
 void launch_accum_v(int mode, const R* psi, const R* V, double* acc, const double* occ,
                     const Tile& t, double c, double gs, long long n3, int touch, R* out, cudaStream_t st) {
   const int threads = 256;
   const unsigned blocks = (unsigned)((n3 / VEC + threads - 1) / threads);
+  if (blocks < kWideBlocks) {
+    const dim3 grid(blocks, t.diag ? t.ti : t.ti + t.tj);
+    k_accum_wide<R, 8, VEC><<<grid, threads, 0, st>>>(psi, V, acc, occ, t.i0, t.ti, t.j0, t.tj, t.diag, c, gs, n3,
+                                                      touch, out);
+    return;
+  }
   auto go = [&](auto k) {
     k<<<blocks, threads, 0, st>>>(psi, V, acc, occ, t.i0, t.ti, t.j0, t.tj, t.diag, c, gs, n3, touch, out);
   };
@@ -683,8 +727,9 @@ exx_status_t exx_plan_info(exx_plan_t p, int* tile, int* ntiles, size_t* workspa
   if (ntiles) *ntiles = nt;
   if (workspace_bytes) *workspace_bytes = p->ws;
   const bool conv = p->vacc != nullptr && p->sharded;  // else part of the accumulation
-  if (launches_apply) *launches_apply = 5 * nt + 1 + (conv ? 1 : 0);
-  if (launches_energy) *launches_energy = 3 * nt + 1;
+  const int total = p->tiles.size() == 1 && p->mine[0] ? 0 : 1;  // a single tile's launch sums E_x too
+  if (launches_apply) *launches_apply = 5 * nt + total + (conv ? 1 : 0);
+  if (launches_energy) *launches_energy = 3 * nt + total;
   return EXX_OK;
 }
 
@@ -726,6 +771,7 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
   // of one accumulator at a time), and a lane overwrites its V only after the
   // accumulation of its previous tile has read it.
   const int nl = p->lanes;
+  const bool single = p->tiles.size() == 1 && p->mine[0];  // pair energies and E_x in one launch
   if (nl > 1) {
     EXX_CUDA(p, cudaEventRecord(p->ev_fork, st));
     for (int l = 0; l < nl; ++l) EXX_CUDA(p, cudaStreamWaitEvent(p->ls[l], p->ev_fork, 0));
@@ -767,7 +813,11 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
       if (p->plane) p->ops->plane(X2, Yt, p->Gs, p->tw, ep, t.count, !apply, sl);
       else p->ops->zconv(X2, p->Gs, p->twz ? p->twz : p->tw, &p->gmap, ep, p->d_err, t.count, !apply, sl);
     }
-    {
+    if (single) {
+      ProfScope ps(p, K_TOTAL, sl);
+      k_pair_energy_total<<<1, 1024, 0, sl>>>(ep, nper, pr, t.count, h3, p->Epair, N, p->d_occ, p->alpha,
+                                              E_dev ? E_dev : p->E_dev);
+    } else {
       ProfScope ps(p, K_PAIRE, sl);
       k_pair_energy<<<(t.count * 32 + 255) / 256, 256, 0, sl>>>(ep, nper, pr, t.count, h3,
                                                                   p->Epair);
@@ -815,7 +865,7 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
       EXX_CUDA(p, cudaEventRecord(p->ev_done[l], p->ls[l]));
       EXX_CUDA(p, cudaStreamWaitEvent(st, p->ev_done[l], 0));
     }
-  {
+  if (!single) {
     ProfScope ps(p, K_TOTAL, st);
     k_exx_total<<<1, 256, 0, st>>>(p->Epair, p->P, N, p->d_occ, p->alpha, E_dev ? E_dev : p->E_dev);
   }
@@ -850,6 +900,10 @@ exx_status_t exx_energy_async(exx_plan_t p, const void* psi, double* E_dev, void
 // A bounded device-side wait that ran out leaves a flag; the synchronising
 // calls report it as EXX_ERR_TIMEOUT (and clear it).
 static exx_status_t check_wait_flag(exx_plan_t p, cudaStream_t st) {
+  if (p->plane) {  // no kernel of the plane pipeline waits on a flag
+    EXX_CUDA(p, cudaStreamSynchronize(st));
+    return EXX_OK;
+  }
   int f = 0;
   EXX_CUDA(p, cudaMemcpyAsync(&f, p->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
   EXX_CUDA(p, cudaStreamSynchronize(st));

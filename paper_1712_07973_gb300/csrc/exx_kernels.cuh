@@ -997,6 +997,74 @@ k_accum(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__
                                TOUCH < 0 ? touch : TOUCH, TOUCH < 0 || (TOUCH & T_LAST_I) ? out : nullptr);
 }
 
+// The same sums, one orbital of the tile per blockIdx.y (block I, then block J),
+// each in accum_tile's order: for small grids, whose points alone leave most SMs
+// idle while every thread walks through the tile's pairs.  Reads each potential
+// twice (from L2).
+template <typename R, int TM, int VEC>
+__global__ void __launch_bounds__(256)
+k_accum_wide(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__ vx,
+             const double* __restrict__ occ, int i0, int ti, int j0, int tj, int diag, double c,
+             double gs, long long n3, int touch, R* out) {
+  const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * VEC;
+  if (r >= n3) return;
+  const int s = blockIdx.y;
+  const bool on_i = s < ti;             // block I's orbital s (diagonal tiles: I = J), else block J's s - ti
+  const int k = on_i ? s : s - ti;
+  const int cnt = on_i ? tj : ti, o0 = on_i ? j0 : i0;  // the other side of k's pairs
+  R v[TM][VEC], q[TM][VEC], f[TM];
+#pragma unroll
+  for (int m = 0; m < TM; ++m) {
+    f[m] = R(0);
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) v[m][e] = q[m][e] = R(0);
+    if (m < cnt) {
+      const int a = on_i && !(diag && m < k) ? k : m, b = on_i && !(diag && m < k) ? m : k;
+      const int slot = diag ? a * tj - (a * (a - 1)) / 2 + (b - a) : a * tj + b;
+      vload<R, VEC>(V + (long long)slot * n3 + r, v[m]);
+      vload<R, VEC>(psi + (long long)(o0 + m) * n3 + r, q[m]);
+      f[m] = (R)occ[o0 + m];
+    }
+  }
+  R acc[VEC];
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) acc[e] = R(0);
+  if (diag) {
+    // accum_tile's order: the pair (k, k), the pairs (m, k) with m < k as one
+    // sum, the pairs (k, m)
+    R lo[VEC];
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) lo[e] = R(0);
+#pragma unroll
+    for (int m = 0; m < TM; ++m)
+      if (m < k) {
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) lo[e] += f[m] * v[m][e] * q[m][e];
+      }
+#pragma unroll
+    for (int m = 0; m < TM; ++m) {
+      if (m < k || m >= cnt) continue;
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) {
+        acc[e] += f[m] * v[m][e] * q[m][e];
+        if (m == k) acc[e] += lo[e];
+      }
+    }
+  } else {
+#pragma unroll
+    for (int m = 0; m < TM; ++m) {
+      if (m >= cnt) break;
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) acc[e] += f[m] * v[m][e] * q[m][e];
+    }
+  }
+  const int ko = (on_i ? i0 : j0) + k;
+  const double ck = gs != 0.0 ? c * (gs * occ[ko]) : c;
+  const long long o = (long long)ko * n3 + r;
+  vacc<R, VEC>(vx + o, ck, acc, (touch & (on_i ? T_FIRST_I : T_FIRST_J)) != 0,
+               on_i && out != nullptr ? out + o : nullptr);
+}
+
 // Tile descriptor of a batched wave (tiles of different molecules, or of
 // disjoint orbital blocks, so that no two touch the same accumulator).
 struct TileDesc {
