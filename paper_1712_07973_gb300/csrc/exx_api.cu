@@ -137,6 +137,7 @@ __host__ __device__ inline void tri_decode(long long g, long long N, int* pi, in
 __global__ void k_pair_energy(const double* __restrict__ epart, int nper,
                               const int4* __restrict__ pairs, int npair, double h3,
                               double* __restrict__ Epair) {
+  dep_wait();
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= npair) return;
@@ -151,6 +152,7 @@ __global__ void k_pair_energy(const double* __restrict__ epart, int nper,
 // (Eq. HF).  One block, fixed-order tree reduction; pairs decoded on device.
 __global__ void k_exx_total(const double* __restrict__ Epair, long long P, int N,
                             const double* __restrict__ occ, double alpha, double* __restrict__ E) {
+  dep_wait();
   __shared__ double red[256];
   double s = 0.0;
   for (long long g = threadIdx.x; g < P; g += blockDim.x) {
@@ -174,6 +176,7 @@ __global__ void __launch_bounds__(1024) k_pair_energy_total(const double* __rest
                                                             const int4* __restrict__ pairs, int npair, double h3,
                                                             double* Epair, int N, const double* __restrict__ occ,
                                                             double alpha, double* __restrict__ E) {
+  dep_wait();
   __shared__ double red[256];
   const int lane = threadIdx.x & 31;
   for (int w = threadIdx.x >> 5; w < npair; w += 32) {
@@ -421,12 +424,13 @@ void launch_accum_v(int mode, const R* psi, const R* V, double* acc, const doubl
   const unsigned blocks = (unsigned)((n3 / VEC + threads - 1) / threads);
   if (blocks < kWideBlocks) {
     const dim3 grid(blocks, t.diag ? t.ti : t.ti + t.tj);
-    k_accum_wide<R, 8, VEC><<<grid, threads, 0, st>>>(psi, V, acc, occ, t.i0, t.ti, t.j0, t.tj, t.diag, c, gs, n3,
-                                                      touch, out);
+    launch_dep(k_accum_wide<R, 8, VEC>, grid, threads, 0, st, psi, V, acc, occ, t.i0, t.ti, t.j0, t.tj, t.diag, c,
+               gs, n3, touch, out);
     return;
   }
   auto go = [&](auto k) {
-    k<<<blocks, threads, 0, st>>>(psi, V, acc, occ, t.i0, t.ti, t.j0, t.tj, t.diag, c, gs, n3, touch, out);
+    launch_dep(k, dim3(blocks), threads, 0, st, psi, V, acc, occ, t.i0, t.ti, t.j0, t.tj, t.diag, c, gs, n3, touch,
+               out);
   };
   auto by_mode = [&](auto T) {
     constexpr int t = decltype(T)::value;
@@ -653,12 +657,14 @@ static exx_status_t plan_create_impl(exx_plan_t* out, const int grid[3], const d
   EXX_ALLOC(p->E_dev, sizeof(double));
   EXX_ALLOC(p->d_err, 2 * sizeof(int));
   // pipeline lanes: two by default (a tile's line kernels, bound by memory, run
-  // beside the other tile's plane kernel: 96^3 8.81 -> 8.50 ms with 32
-  // orbitals), one where the slab kernels run as CTA clusters; EXX_LANES=1..3 at plan creation chooses; never more than the
+  // beside the other tile's plane kernel: 96^3 8.33 -> 8.15 ms with 32
+  // orbitals), one where the planes go through in halves (160^3 24 orbitals 25.7
+  // ms with one lane, 26.4 with two; 128^3 12.5 and 12.65) or the slab kernels run
+  // as CTA clusters; EXX_LANES=1..3 at plan creation chooses; never more than the
   // plan has tiles
   {
     const char* env = std::getenv("EXX_LANES");
-    int nl = ops->clustered && !p->plane ? 1 : kDefaultLanes;
+    int nl = (p->plane ? ops->plane_ry == 2 : ops->clustered) ? 1 : kDefaultLanes;
     if (env && env[0] >= '1' && env[0] <= '0' + kMaxLanes && env[1] == '\0') nl = env[0] - '0';
     p->max_lanes = p->lanes = (int)std::min<size_t>((size_t)nl, p->tiles.size());
   }
@@ -813,15 +819,18 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
       if (p->plane) p->ops->plane(X2, Yt, p->Gs, p->tw, ep, t.count, !apply, sl);
       else p->ops->zconv(X2, p->Gs, p->twz ? p->twz : p->tw, &p->gmap, ep, p->d_err, t.count, !apply, sl);
     }
-    if (single) {
-      ProfScope ps(p, K_TOTAL, sl);
-      k_pair_energy_total<<<1, 1024, 0, sl>>>(ep, nper, pr, t.count, h3, p->Epair, N, p->d_occ, p->alpha,
-                                              E_dev ? E_dev : p->E_dev);
-    } else {
-      ProfScope ps(p, K_PAIRE, sl);
-      k_pair_energy<<<(t.count * 32 + 255) / 256, 256, 0, sl>>>(ep, nper, pr, t.count, h3,
-                                                                  p->Epair);
-    }
+    // (behind the inverse transforms, which do not wait for it)
+    auto energies = [&]() {
+      if (single) {
+        ProfScope ps(p, K_TOTAL, sl);
+        launch_dep(k_pair_energy_total, dim3(1), 1024, 0, sl, ep, nper, pr, t.count, h3, p->Epair, N, p->d_occ,
+                   p->alpha, E_dev ? E_dev : p->E_dev);
+      } else {
+        ProfScope ps(p, K_PAIRE, sl);
+        launch_dep(k_pair_energy, dim3((t.count * 32 + 255) / 256), 256, 0, sl, ep, nper, pr, t.count, h3, p->Epair);
+      }
+    };
+    if (!apply) energies();
     if (apply) {
       // vector width: 4 (FP32) or 2 values per thread when n^3 and the
       // caller's pointers allow aligned vector accesses
@@ -847,6 +856,7 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
         EXX_CUDA(p, cudaStreamWaitEvent(st, p->ev_done[l], 0));
       }
       used[l] = true;
+      energies();
       {
         ProfScope ps(p, K_ACCUM, st);
         if (p->prec == EXX_FP64)
@@ -867,7 +877,7 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
     }
   if (!single) {
     ProfScope ps(p, K_TOTAL, st);
-    k_exx_total<<<1, 256, 0, st>>>(p->Epair, p->P, N, p->d_occ, p->alpha, E_dev ? E_dev : p->E_dev);
+    launch_dep(k_exx_total, dim3(1), 256, 0, st, p->Epair, p->P, N, p->d_occ, p->alpha, E_dev ? E_dev : p->E_dev);
   }
   if (apply && p->vacc && p->sharded) {
     ProfScope ps(p, K_CONV, st);

@@ -352,8 +352,11 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
         g.ops->fwd_xy(nullptr, psi_tab, pr, w.npair, Xl[l], g.tw, n3, sl);
         g.ops->zconv(Xl[l], g.Gs, g.tw, &g.gmap, epl[l], b->d_err, w.npair, !apply, sl);
       }
-      k_pair_energy<<<(w.npair * 32 + 255) / 256, 256, 0, sl>>>(epl[l], nper, pr, w.npair, h3,
-                                                                 b->Epair);
+      // (behind the inverse transforms, which do not wait for it)
+      auto energies = [&]() {
+        launch_dep(k_pair_energy, dim3((w.npair * 32 + 255) / 256), 256, 0, sl, epl[l], nper, pr, w.npair, h3, b->Epair);
+      };
+      if (!apply) energies();
       if (apply) {
         if (nl > 1 && used[l] && cudaStreamWaitEvent(sl, b->ev_free[l], 0) != cudaSuccess)
           return EXX_ERR_CUDA;
@@ -363,18 +366,14 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
                        cudaStreamWaitEvent(st, b->ev_done[l], 0) != cudaSuccess))
           return EXX_ERR_CUDA;
         used[l] = true;
+        energies();
         float* const* out = b->persistent ? nullptr : b->d_vx_tab;
         const bool v2 = b->vec2 && (n3 % 2) == 0;
         const int threads = 256;
         const long long blocks = (n3 / (v2 ? 2 : 1) + threads - 1) / threads;
-        if (v2)
-          k_accum_batch<float, 8, 2><<<dim3((unsigned)blocks, w.ntile), threads, 0, st>>>(
-              b->d_psi_tab, static_cast<const float*>(Vl[l]), b->d_vacc_tab, out, b->d_occ,
-              b->d_tiles + w.tile_off, grad ? 1 : 0, n3);
-        else
-          k_accum_batch<float, 8, 1><<<dim3((unsigned)blocks, w.ntile), threads, 0, st>>>(
-              b->d_psi_tab, static_cast<const float*>(Vl[l]), b->d_vacc_tab, out, b->d_occ,
-              b->d_tiles + w.tile_off, grad ? 1 : 0, n3);
+        launch_dep(v2 ? k_accum_batch<float, 8, 2> : k_accum_batch<float, 8, 1>, dim3((unsigned)blocks, w.ntile),
+                   threads, 0, st, b->d_psi_tab, static_cast<const float*>(Vl[l]), b->d_vacc_tab, out, b->d_occ,
+                   b->d_tiles + w.tile_off, grad ? 1 : 0, n3);
         if (nl > 1 && cudaEventRecord(b->ev_free[l], st) != cudaSuccess) return EXX_ERR_CUDA;
       }
     }

@@ -88,6 +88,14 @@ template <int P, bool FULL, typename C> EXX_HD void dft_inv_out(C* v) {
   else dft_halfout<P, 1>(v);
 }
 
+// Programmatic dependent launch: a kernel launched with launch_dep (exx_ops.cuh)
+// may start while the one ahead of it in its stream drains; dep_wait waits for
+// that one's results (and for those it waited for itself), so it comes before
+// the first access to anything a kernel writes.  (No launch_dependents: CTAs
+// that start earlier and hold their share of an SM while they wait cost 2% at
+// 160^3 and 20% of an FP64 call on 32^3.)
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
 // Tensor-memory-access (TMA) load with an mbarrier (PTX, sm_90 and later).
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
   return (unsigned)__cvta_generic_to_shared(p);
@@ -991,6 +999,7 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && MODE == 0) ? 3 : 2)
 k_accum(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__ vx,
         const double* __restrict__ occ, int i0, int ti, int j0, int tj, int diag, double c,
         double gs, long long n3, int touch, R* out) {
+  dep_wait();
   const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * VEC;
   if (r >= n3) return;
   accum_tile<R, TM, VEC, MODE>(psi, V, vx, occ, i0, ti, j0, tj, diag, c, gs, n3, r,
@@ -1006,6 +1015,7 @@ __global__ void __launch_bounds__(256)
 k_accum_wide(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__ vx,
              const double* __restrict__ occ, int i0, int ti, int j0, int tj, int diag, double c,
              double gs, long long n3, int touch, R* out) {
+  dep_wait();
   const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * VEC;
   if (r >= n3) return;
   const int s = blockIdx.y;
@@ -1115,6 +1125,7 @@ __global__ void __launch_bounds__(256, 2)
 k_accum_batch(const R* const* __restrict__ psi_tab, const R* __restrict__ V,
               double* const* __restrict__ vx_tab, R* const* __restrict__ vx_out,
               const double* __restrict__ occ, const TileDesc* __restrict__ tiles, int grad, long long n3) {
+  dep_wait();
   accum_batch_unit<R, TM, VEC, false>(psi_tab, V, vx_tab, vx_out, occ, tiles, grad, n3, blockIdx.x,
                                       blockIdx.y, blockDim.x);
 }

@@ -147,6 +147,25 @@ inline bool make_ktab_map(CUtensorMap* map, const void* table, int n, int nz) {
                 CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Launch that may start before the kernel ahead of it in the stream has finished
+// (programmatic dependent launch): only for kernels that call dep_wait.  On the
+// device, per call: 5 orbitals 24^3 33.7 -> 21.9 us, FP64 4 orbitals 32^3 238 -> 226,
+// 16 orbitals 64^3 651 -> 643.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_dep(void (*kern)(KArgs...), dim3 grid, int nt, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(nt);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
 // Launch of a slab kernel; CL > 1 launches (CL, 1, 1) thread-block clusters.
 template <int CL, typename... KArgs, typename... Args>
 inline void launch_slab(void (*kern)(KArgs...), dim3 grid, int nt, size_t smem, cudaStream_t st,
@@ -436,9 +455,8 @@ template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> stru
   static void xfwd(const void* psi, const void* const* psi_tab, const int4* pairs, int npair, void* X, const void* tw,
                    long long n3, cudaStream_t st) {
     if constexpr (plane_ok)
-      k_xfwd<R, N, PER><<<dim3(npair * XC::NZB, G), XC::NT, XC::smem_f, st>>>(
-          static_cast<const R*>(psi), reinterpret_cast<const R* const*>(psi_tab), pairs, static_cast<C*>(X),
-          static_cast<const C*>(tw), n3);
+      launch_dep(k_xfwd<R, N, PER>, dim3(npair * XC::NZB, G), XC::NT, XC::smem_f, st, static_cast<const R*>(psi),
+                 reinterpret_cast<const R* const*>(psi_tab), pairs, static_cast<C*>(X), static_cast<const C*>(tw), n3);
   }
   static void plane(const void* X, void* Y, const void* Gs, const void* tw, double* epart, int npair, bool energy_only,
                     cudaStream_t st) {
@@ -446,14 +464,14 @@ template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> stru
       const int planes = npair * (N + 1), full = 152 * PC::MINB;
       const int grid = planes < full ? planes : full;
       auto k = energy_only ? plk<true>() : plk<false>();
-      k<<<grid, PC::NT, PC::smem, st>>>(static_cast<const C*>(X), static_cast<C*>(Y), static_cast<const R*>(Gs),
-                                        static_cast<const C*>(tw) + 3 * N, epart, npair, N + 1);
+      launch_dep(k, dim3(grid), PC::NT, PC::smem, st, static_cast<const C*>(X), static_cast<C*>(Y),
+                 static_cast<const R*>(Gs), static_cast<const C*>(tw) + 3 * N, epart, npair, N + 1);
     }
   }
   static void xinv(const void* X, void* V, const void* tw, int npair, cudaStream_t st) {
     if constexpr (plane_ok)
-      k_xinv<R, N, PER><<<dim3(npair * XC::NZB, G), XC::NT, XC::smem_i, st>>>(
-          static_cast<const C*>(X), static_cast<R*>(V), static_cast<const C*>(tw));
+      launch_dep(k_xinv<R, N, PER>, dim3(npair * XC::NZB, G), XC::NT, XC::smem_i, st, static_cast<const C*>(X),
+                 static_cast<R*>(V), static_cast<const C*>(tw));
   }
 
   // gains of the x and y transforms, and of the z transform

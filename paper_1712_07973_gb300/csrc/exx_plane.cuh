@@ -268,6 +268,7 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     stash = tslot + ((unsigned)(warp & 3) << 21) + (unsigned)(warp >> 2) * (K::ZROUNDS * K::WST);
   }
+  dep_wait();
   const int nplane = npair * nkx;
   // plane pl: kx = pl / npair, pair pl % npair (the pairs of one kx together:
   // its kernel-table rows stay in L2)
@@ -621,6 +622,7 @@ k_xfwd(const R* __restrict__ psi0, const R* const* __restrict__ psi_tab, const i
   const R* psi = psi_tab ? psi_tab[pr.w] : psi0;
   const R* __restrict__ pi = psi + (long long)pr.x * n3 + (long long)z0 * G * G + y * G;
   const R* __restrict__ pj = psi + (long long)pr.y * n3 + (long long)z0 * G * G + y * G;
+  dep_wait();
   // rho[2m] + i rho[2m+1], whole rows; paired loads where the caller's orbitals
   // are aligned for them
   if ((reinterpret_cast<size_t>(psi) & (sizeof(C) - 1)) == 0) {
@@ -758,6 +760,7 @@ k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restri
     }
     if (q == 0) xn = __ldcs(&in[(long long)N * KS].x);
   };
+  dep_wait();
   if (tid < K::UB) load(tid);
   for (int t = tid; t < 2 * N; t += NT) tw[t] = tw_g[t];
   __syncthreads();
