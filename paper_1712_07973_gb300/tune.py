@@ -11,7 +11,6 @@ and keeps the fastest in a JSON cache keyed by (n, N, precision, SM count);
 
 import json
 import os
-import statistics
 
 __all__ = ["CANDIDATES", "cache_path", "cache_key", "load_cache", "store", "best_tile", "tune"]
 
@@ -66,9 +65,16 @@ def best_tile(n, N, precision="fp32", tune_if_missing=False, path=None):
     return 0
 
 
+# timings this close are ties: small molecules are bound by their launches, whose
+# times scatter by a few per cent from one process to the next
+TIE = 0.10
+
+
 def select(timings):
-    """Fastest candidate; ties go to the larger tile (less accumulator traffic)."""
-    return min(timings, key=lambda t: (timings[t], -t))
+    """Fastest candidate; ties (within TIE of the fastest) go to the larger tile
+    (less accumulator traffic)."""
+    most = (1.0 + TIE) * min(timings.values())
+    return max(t for t in timings if timings[t] <= most)
 
 
 def tune(n, N, precision="fp32", h=0.4, reps=3, candidates=CANDIDATES, path=None, measure=None,
@@ -102,18 +108,22 @@ def _gpu_measure(n, N, precision, h, reps):
     def measure(tile):
         plan = exx.ExxPlan(n, h, 0.25, occ, precision=precision, tile=tile)
         out = torch.empty(psi.shape, dtype=plan.vx_dtype, device=psi.device)
-        plan.apply_async(psi, out)
-        torch.cuda.synchronize()
-        times = []
-        for _ in range(reps):
+        def timed(calls):
             a = torch.cuda.Event(enable_timing=True)
             b = torch.cuda.Event(enable_timing=True)
             a.record()
-            plan.apply_async(psi, out)
+            for _ in range(calls):
+                plan.apply_async(psi, out)
             b.record()
             torch.cuda.synchronize()
-            times.append(a.elapsed_time(b))
+            return a.elapsed_time(b) / calls
+
+        plan.apply_async(psi, out)
+        torch.cuda.synchronize()
+        # short calls: a few milliseconds of them per repetition
+        calls = max(1, min(64, int(4.0 / max(timed(1), 1e-3))))
+        times = [timed(calls) for _ in range(reps)]
         plan.close()
-        return statistics.median(times)
+        return min(times)
 
     return measure
