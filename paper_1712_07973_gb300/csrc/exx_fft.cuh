@@ -172,6 +172,52 @@ template <int SIGN, int P, int E, typename C> EXX_HD C twmul(C a) {
   }
 }
 
+// a + k u for a constant k, lane by lane (one multiply-add per lane; FP32 on the
+// device: one packed instruction)
+template <typename C> EXX_HD C caxpy(C a, double k, C u) {
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+  if constexpr (std::is_same<C, float2>::value) return __ffma2_rn(u, make_float2((float)k, (float)k), a);
+#endif
+  return mkc<C>(kfma(u.x, k, a.x), kfma(u.y, k, a.y));
+}
+// omega^E = k (1 + i t) for an odd multiple of pi/4 (t = +-1, |k| = 1/sqrt2): the
+// factor k is left to the sum that follows, b (1 + i t) here
+template <int SIGN, int P, int E> struct eighth {
+  static constexpr long e = pmod(E, P);
+  static constexpr bool is = 8 * e == P || 8 * e == 3 * P || 8 * e == 5 * P || 8 * e == 7 * P;
+  static constexpr bool cp = cos2pi(E, P) > 0, sp = (SIGN * sin2pi(E, P)) > 0;
+  static constexpr double k = cp ? 0.70710678118654752440084436210485 : -0.70710678118654752440084436210485;
+  template <typename C> static EXX_HD C part(C b) {
+    return cp == sp ? mkc<C>(b.x - b.y, b.y + b.x) : mkc<C>(b.x + b.y, b.y - b.x);
+  }
+};
+// a + omega^E b, the product folded into the sum (four multiply-adds instead of
+// four and two additions; two additions and two multiply-adds for odd multiples
+// of pi/4)
+template <int SIGN, int P, int E, typename C> EXX_HD C twadd(C a, C b) {
+  constexpr long e = pmod(E, P);
+  if constexpr (4 * e % P == 0) {
+    return cadd(a, twmul<SIGN, P, E>(b));
+  } else if constexpr (eighth<SIGN, P, E>::is) {
+    return caxpy(a, eighth<SIGN, P, E>::k, eighth<SIGN, P, E>::part(b));
+  } else {
+    constexpr double c = cos2pi(E, P), s = SIGN * sin2pi(E, P);
+    return mkc<C>(kfma(b.x, c, kfma(b.y, -s, a.x)), kfma(b.x, s, kfma(b.y, c, a.y)));
+  }
+}
+// p = a + omega^E b, m = a - omega^E b
+template <int SIGN, int P, int E, typename C> EXX_HD void twbfly(C a, C b, C& p, C& m) {
+  if constexpr (eighth<SIGN, P, E>::is) {
+    const C u = eighth<SIGN, P, E>::part(b);
+    p = caxpy(a, eighth<SIGN, P, E>::k, u);
+    m = caxpy(a, -eighth<SIGN, P, E>::k, u);
+  } else {
+    const C t = twmul<SIGN, P, E>(b);
+    p = cadd(a, t);
+    m = csub(a, t);
+  }
+}
+
 // ------------------------------------------------------------ DFT kernels
 // v[S*i], i < P : in-place DFT, natural order in and out.
 
@@ -199,10 +245,10 @@ template <int S, int SIGN, typename C> EXX_HD void dft3(C* v) {
   C t1 = cadd(b, c);
   C t2 = mkc<C>(a.x - R(0.5) * t1.x, a.y - R(0.5) * t1.y);
   C d = csub(b, c);
-  C t3 = mkc<C>(-kmul(d.y, s3), kmul(d.x, s3));  // i * s3 * (b - c)
   v[0] = cadd(a, t1);
-  v[S] = cadd(t2, t3);
-  v[2 * S] = csub(t2, t3);
+  // t2 +- i s3 (b - c)
+  v[S] = mkc<C>(kfma(d.y, -s3, t2.x), kfma(d.x, s3, t2.y));
+  v[2 * S] = mkc<C>(kfma(d.y, s3, t2.x), kfma(d.x, -s3, t2.y));
 }
 
 template <int S, int SIGN, typename C> EXX_HD void dft4(C* v) {
@@ -244,6 +290,51 @@ template <int P, int S, int SIGN, typename C> EXX_HD void dft_prime(C* v) {
     v[(P - k) * S] = mkc<C>(re - qre, im - qim);
   });
   v[0] = tot;
+}
+
+// P = 8: the length-4 DFTs of the even and the odd samples, then the butterflies
+// with their rotations by odd multiples of pi/4 folded in.
+template <int S, int SIGN, typename C> EXX_HD void dft8(C* v) {
+  dft4<2 * S, SIGN>(v);      // even samples: E[k] at 2k
+  dft4<2 * S, SIGN>(v + S);  // odd samples: O[k] at 2k + 1
+  C p[4], m[4];
+  sfor<4>([&](auto K) { twbfly<SIGN, 8, (int)K>(v[2 * K * S], v[(2 * K + 1) * S], p[K], m[K]); });
+  sfor<4>([&](auto K) {
+    v[K * S] = p[K];
+    v[(K + 4) * S] = m[K];
+  });
+}
+
+// P = 16 = 4 x 4: first DFTs over n1 (n = 4 n1 + n2), rotations by w^(n2 k1), DFTs
+// over n2; where two partners of a butterfly are both rotated by odd multiples
+// of pi/4 (k1 = 2), the common 1/sqrt2 goes to the last sums.
+template <int S, int SIGN, typename C> EXX_HD void dft16(C* v) {
+  sfor<4>([&](auto N2) { dft4<4 * S, SIGN>(v + N2 * S); });  // X[n2][k1] at 4 k1 + n2
+  C t[16];
+  sfor<4>([&](auto K1) {
+    constexpr int k1 = K1;
+    const C a = v[(4 * k1) * S], b = v[(4 * k1 + 1) * S], c = v[(4 * k1 + 2) * S], d = v[(4 * k1 + 3) * S];
+    C s0, s1;
+    twbfly<SIGN, 16, 2 * k1>(a, c, s0, s1);
+    if constexpr (k1 == 2) {
+      // w^2 and w^6 = SIGN i w^2: r (B +- D) with B = b (1 + SIGN i), D = SIGN i d (1 + SIGN i)
+      constexpr double r = eighth<SIGN, 16, 2>::k;
+      const C B = eighth<SIGN, 16, 2>::part(b), D = mul_si<SIGN>(eighth<SIGN, 16, 2>::part(d));
+      const C q0 = cadd(B, D), q1 = mul_si<SIGN>(csub(B, D));
+      t[k1] = caxpy(s0, r, q0);
+      t[k1 + 8] = caxpy(s0, -r, q0);
+      t[k1 + 4] = caxpy(s1, r, q1);
+      t[k1 + 12] = caxpy(s1, -r, q1);
+    } else {
+      const C B = twmul<SIGN, 16, k1>(b), D = twmul<SIGN, 16, 3 * k1>(d);
+      const C s2 = cadd(B, D), s3 = mul_si<SIGN>(csub(B, D));
+      t[k1] = cadd(s0, s2);
+      t[k1 + 8] = csub(s0, s2);
+      t[k1 + 4] = cadd(s1, s3);
+      t[k1 + 12] = csub(s1, s3);
+    }
+  });
+  sfor<16>([&](auto I) { v[I * S] = t[I]; });
 }
 
 // composite P = A * B (A = first factor): input n = B*n1 + n2, output k1 + A*k2
@@ -316,7 +407,9 @@ template <int P, int S, int SIGN, typename C> EXX_HD void dft(C* v) {
     dft_prime<P, S, SIGN>(v);
   } else {
     static_assert(first_factor<P>::value != P, "DFT length with a prime factor > 7");
-    if constexpr (pfa_a(P) != P) dft_pfa<P, S, SIGN>(v);  // coprime factors
+    if constexpr (P == 8) dft8<S, SIGN>(v);
+    else if constexpr (P == 16) dft16<S, SIGN>(v);
+    else if constexpr (pfa_a(P) != P) dft_pfa<P, S, SIGN>(v);  // coprime factors
     else dft_composite<P, S, SIGN>(v);                     // a prime power
   }
 }
@@ -351,7 +444,7 @@ template <int P, int SIGN, typename C> EXX_HD void dft_halfout(C* v) {
   });
   dft<H, 1, SIGN>(e);
   dft<H, 1, SIGN>(o);
-  sfor<H>([&](auto J) { v[J] = cadd(e[J], twmul<SIGN, P, (int)J>(o[J])); });
+  sfor<H>([&](auto J) { v[J] = twadd<SIGN, P, (int)J>(e[J], o[J]); });
 }
 
 // Four-step split of a line length L = L1 * L2: L1 even (pruning), L1 <= 16,

@@ -462,7 +462,7 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
 #pragma unroll
               for (int k = 0; k < ZH; ++k) v[k] = o[ZL2 * k];
               dft<ZH, 1, 1>(v);
-              sfor<ZH>([&](auto J) { o[ZL2 * J] = cadd(a[J], twmul<1, ZL1, (int)J>(v[J])); });
+              sfor<ZH>([&](auto J) { o[ZL2 * J] = twadd<1, ZL1, (int)J>(a[J], v[J]); });
             }
           }
           __syncthreads();
@@ -532,13 +532,13 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
             }
             dft<YH, 1, 1>(e);
             dft<YH, 1, 1>(v);
-            sfor<YH>([&](auto J) { q[YL2 * J * G] = cadd(e[J], twmul<1, YL1, (int)J>(v[J])); });
+            sfor<YH>([&](auto J) { q[YL2 * J * G] = twadd<1, YL1, (int)J>(e[J], v[J]); });
           } else {
 #pragma unroll
             for (int k = 0; k < YH; ++k) v[k] = o[k * ZP];
             dft<YH, 1, 1>(v);
             if (sy) {
-              sfor<YH>([&](auto J) { v[J] = cadd(na[J], twmul<1, YL1, (int)J>(v[J])); });
+              sfor<YH>([&](auto J) { v[J] = twadd<1, YL1, (int)J>(na[J], v[J]); });
               fetch_a(u + NTG);
             }
 #pragma unroll
