@@ -283,8 +283,8 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
   // launch per pass: every orbital's first update clears and its last converts
   // (TileDesc::touch); the persistent queue clears and converts in passes
   if (apply && b->persistent) {
-    long long tot = 0;
-    for (const Mol& m : b->mol) tot += (long long)m.N * m.n * m.n * m.n;
+    const Mol& last = b->mol.back();
+    const long long tot = last.vacc_off + (long long)last.N * last.n * last.n * last.n;
     if (cudaMemsetAsync(b->vacc, 0, (size_t)tot * sizeof(double), st) != cudaSuccess) return EXX_ERR_CUDA;
   }
   // two lanes: consecutive waves alternate between two streams with their own
@@ -507,7 +507,7 @@ exx_status_t exx_batch_create(exx_batch_t* out, int nmol, const exx_mol_desc* mo
     mm.ep_off = ep;
     ep += mm.P;
     mm.vacc_off = vo;
-    vo += (long long)d.norb * d.n * d.n * d.n;
+    vo += ((long long)d.norb * d.n * d.n * d.n + 3) / 4 * 4;  // each molecule's accumulators stay 32-byte aligned
     mm.group = -1;
     for (size_t g = 0; g < b->groups.size(); ++g)
       if (b->groups[g].n == d.n && b->groups[g].h == d.h) mm.group = (int)g;

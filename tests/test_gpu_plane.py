@@ -44,3 +44,29 @@ def test_plane_pipeline_against_oracle(bc, n, prec):
     assert abs(E - Eo) <= e_tol and abs(Ee - Eo) <= e_tol
     assert np.max(np.abs(Eij - [Eijo[0, 0], Eijo[0, 1], Eijo[1, 1]])) <= e_tol
     assert np.max(np.abs(vx.double().cpu().numpy() - vxo)) <= v_tol
+
+
+@pytest.mark.parametrize("persistent", [False, True])
+def test_batch_with_an_odd_number_of_accumulators_before_even_grids(persistent):
+    # 3 orbitals on 9^3 hold an odd number of FP64 accumulators; those of the
+    # next molecules (vector accesses) must stay aligned
+    import torch
+    from paper_1712_07973_gb300 import exx
+    dev = torch.device("cuda:0")
+    mols, psis, ref = [], [], []
+    for k, (n, N) in enumerate(((9, 3), (8, 2), (16, 3), (9, 1), (20, 2))):
+        r = synth.OrbitalRecipe(n=n, h=0.45, norb=N, nsites=2, seed=40 + k, gauss_per_orb=3,
+                                sigma=(0.12 * n * 0.45, 0.2 * n * 0.45), p_type=True)
+        psis.append(torch.from_numpy(synth.make_orbitals(r)).to(dev, torch.float32))
+        mols.append({"n": n, "h": 0.45, "alpha": 0.25, "occupations": np.full(N, 2.0)})
+        Gh = o.kernel_spectrum(o.kernel_real_space(n, 0.45))
+        ref.append(o.exx(psis[-1].double().cpu().numpy(), np.full(N, 2.0), 0.25, 0.45, Gh)[:2])
+    b = exx.ExxBatch(mols)
+    b.persistent(persistent)
+    vx = [torch.empty_like(p) for p in psis]
+    b.set_buffers(psis, vx)
+    E = b.apply().cpu()
+    for k, (Eo, vo) in enumerate(ref):
+        assert abs(float(E[k]) - Eo) <= 1e-6
+        assert np.max(np.abs(vx[k].double().cpu().numpy() - vo)) <= 2e-6 * np.max(np.abs(vo))
+    b.close()
