@@ -412,15 +412,15 @@ int default_tile(int N, int requested) {
 
 }  // namespace
 
-// Below this many CTAs of points (152 SMs) one orbital per CTA row: 24^3 5 orbitals
-// 16 -> 6 us, 48^3 0.46 -> 0.41 us per pair, 56^3 (172 CTAs) 0.88 -> 0.70; 64^3 (256
+// Below this many CTAs of points (152 SMs, four each) one orbital per CTA row: 24^3 5 orbitals
+// 16 -> 6 us, 48^3 0.46 -> 0.41 us per pair, 56^3 (343 CTAs) 0.88 -> 0.70; 64^3 (512
 // CTAs) 0.71 -> 0.77, its potentials read twice.
-constexpr unsigned kWideBlocks = 200;
+constexpr unsigned kWideBlocks = 400;
 // k_accum launch: vector width 2 when aligned, full-tile specialisations
 template <typename R, int VEC>
 void launch_accum_v(int mode, const R* psi, const R* V, double* acc, const double* occ,
                     const Tile& t, double c, double gs, long long n3, int touch, R* out, cudaStream_t st) {
-  const int threads = 256;
+  const int threads = kAccumThreads;
   const unsigned blocks = (unsigned)((n3 / VEC + threads - 1) / threads);
   if (blocks < kWideBlocks) {
     const dim3 grid(blocks, t.diag ? t.ti : t.ti + t.tj);

@@ -145,6 +145,7 @@ struct exx_batch_s {
   long long* d_count = nullptr;
   bool have_vx = false;
   bool buffers_set = false;
+  bool vec4 = true;  // every orbital and output array 16-byte aligned: loads and stores of four
   bool vec2 = true;  // every orbital array 8-byte aligned: paired loads in accum
   // second pipeline lane (as in a single plan): its workspaces, streams, events
   int lanes = 1;
@@ -368,11 +369,13 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
         used[l] = true;
         energies();
         float* const* out = b->persistent ? nullptr : b->d_vx_tab;
-        const bool v2 = b->vec2 && (n3 % 2) == 0;
-        const int threads = 256;
-        const long long blocks = (n3 / (v2 ? 2 : 1) + threads - 1) / threads;
-        launch_dep(v2 ? k_accum_batch<float, 8, 2> : k_accum_batch<float, 8, 1>, dim3((unsigned)blocks, w.ntile),
-                   threads, 0, st, b->d_psi_tab, static_cast<const float*>(Vl[l]), b->d_vacc_tab, out, b->d_occ,
+        const int vec = b->vec4 && (n3 % 4) == 0 ? 4 : b->vec2 && (n3 % 2) == 0 ? 2 : 1;
+        const int threads = kAccumThreads;
+        const long long blocks = (n3 / vec + threads - 1) / threads;
+        launch_dep(vec == 4   ? k_accum_batch<float, 8, 4>
+                   : vec == 2 ? k_accum_batch<float, 8, 2>
+                              : k_accum_batch<float, 8, 1>,
+                   dim3((unsigned)blocks, w.ntile), threads, 0, st, b->d_psi_tab, static_cast<const float*>(Vl[l]), b->d_vacc_tab, out, b->d_occ,
                    b->d_tiles + w.tile_off, grad ? 1 : 0, n3);
         if (nl > 1 && cudaEventRecord(b->ev_free[l], st) != cudaSuccess) return EXX_ERR_CUDA;
       }
@@ -697,8 +700,12 @@ exx_status_t exx_batch_set_buffers(exx_batch_t b, const float* const* psi, float
     return EXX_ERR_CUDA;
   }
   bool v2 = true;
-  for (int m = 0; m < b->nmol; ++m) v2 = v2 && ((uintptr_t)p[m] % 8 == 0);
-  if (v2 != b->vec2 || have != b->have_vx) {  // the captured graphs embed these choices
+  bool v4 = true;
+  for (int m = 0; m < b->nmol; ++m) {
+    v2 = v2 && ((uintptr_t)p[m] % 8 == 0);
+    v4 = v4 && ((uintptr_t)p[m] % 16 == 0) && ((uintptr_t)v[m] % 16 == 0);
+  }
+  if (v2 != b->vec2 || v4 != b->vec4 || have != b->have_vx) {  // the captured graphs embed these choices
     for (int k = 0; k < 3; ++k)
       if (b->gexec[k]) {
         cudaGraphExecDestroy(b->gexec[k]);
@@ -706,6 +713,7 @@ exx_status_t exx_batch_set_buffers(exx_batch_t b, const float* const* psi, float
       }
   }
   b->vec2 = v2;
+  b->vec4 = v4;
   b->have_vx = have;
   b->buffers_set = true;
   return EXX_OK;

@@ -1,4 +1,8 @@
-// CUDA kernels of the exact-exchange pair pipeline (sm_103a).
+// CUDA kernels of the exact-exchange pair pipeline (sm_103a): the slab pipeline
+// and the accumulation.  Most grids run the plane pipeline of exx_plane.cuh with
+// this file's accumulation; the slab kernels run those it is not built for
+// (FP64 128^3 and 160^3, periodic 192^3, grids below 16 points), the persistent
+// batched kernel and the allocation-free entry point.
 //
 // For every orbital pair (i, j) of a pair tile (arXiv 1712.07973, Sec. 2.1:
 // kernel 1 co-density, kernel 2 Poisson solve, kernel 3 products):
@@ -880,6 +884,22 @@ __device__ __forceinline__ void vload(const R* p, R (&v)[VEC]) {
     for (int e = 0; e < VEC; ++e) v[e] = q[e];
   }
 }
+// The potentials are read once: marked evict-first, so that the orbitals and
+// accumulators stay in L2 (COH: through L2, written in the same launch).
+template <typename R, int VEC, bool COH = false>
+__device__ __forceinline__ void vstream(const R* p, R (&v)[VEC]) {
+  if constexpr (COH) {
+    vload<R, VEC, true>(p, v);
+  } else if constexpr (VEC == 1) {
+    v[0] = __ldcs(p);
+  } else {
+    using V = typename vecty<R, VEC>::type;
+    const V t = __ldcs(reinterpret_cast<const V*>(p));
+    const R* q = reinterpret_cast<const R*>(&t);
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) v[e] = q[e];
+  }
+}
 // vx[0..VEC) += c * a  (FP64); first: the accumulator counts as zero and is
 // not read; out != null: the sum goes there in the working precision (the
 // orbital's last update), not back to the accumulator.  The same sums, bit for
@@ -966,7 +986,7 @@ __device__ __forceinline__ void accum_tile(const R* __restrict__ psi, const R* _
       if (a >= ti || (diag && a > b)) continue;
       const int slot = diag ? a * tj - (a * (a - 1)) / 2 + (b - a) : a * tj + b;
       R v[VEC];
-      vload<R, VEC, COH>(V + (long long)slot * n3 + r, v);
+      vstream<R, VEC, COH>(V + (long long)slot * n3 + r, v);
 #pragma unroll
       for (int e = 0; e < VEC; ++e) {
         ai[a][e] += fb * v[e] * pb[e];
@@ -994,8 +1014,12 @@ __device__ __forceinline__ void accum_tile(const R* __restrict__ psi, const R* _
 // TOUCH: the tile's Touch bits at compile time (a branch around an accumulator's
 // load keeps it from being issued ahead: 1.90 -> 2.16 us per pair at 96^3), or -1:
 // given by touch.
+// CTAs of 128 threads, the registers of 512 (768 in the ragged form) per SM; with
+// the potentials marked evict-first: full FP32 tiles 0.66 -> 0.58 us per pair at
+// 64^3, 1.94 -> 1.85 at 96^3 (4.3 TB/s), 8.4 -> 8.0 at 160^3.
+constexpr int kAccumThreads = 128;
 template <typename R, int TM, int VEC, int MODE, int TOUCH>
-__global__ void __launch_bounds__(256, (sizeof(R) == 4 && MODE == 0) ? 3 : 2)
+__global__ void __launch_bounds__(kAccumThreads, (sizeof(R) == 4 && MODE == 0) ? 6 : 4)
 k_accum(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__ vx,
         const double* __restrict__ occ, int i0, int ti, int j0, int tj, int diag, double c,
         double gs, long long n3, int touch, R* out) {
@@ -1011,7 +1035,7 @@ k_accum(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__
 // idle while every thread walks through the tile's pairs.  Reads each potential
 // twice (from L2).
 template <typename R, int TM, int VEC>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kAccumThreads)
 k_accum_wide(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__ vx,
              const double* __restrict__ occ, int i0, int ti, int j0, int tj, int diag, double c,
              double gs, long long n3, int touch, R* out) {
@@ -1121,7 +1145,7 @@ __device__ __forceinline__ void accum_batch_unit(const R* const* __restrict__ ps
 }
 
 template <typename R, int TM, int VEC>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(kAccumThreads, 4)
 k_accum_batch(const R* const* __restrict__ psi_tab, const R* __restrict__ V,
               double* const* __restrict__ vx_tab, R* const* __restrict__ vx_out,
               const double* __restrict__ occ, const TileDesc* __restrict__ tiles, int grad, long long n3) {

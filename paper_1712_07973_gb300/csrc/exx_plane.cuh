@@ -14,6 +14,12 @@
 // The padded (y, z) part of a spectrum never reaches memory: per pair X (8 n^3
 // bytes in FP32) is written and read twice, where spectra X[kx][z][ky] padded
 // along y move twice that four times.
+//
+// What bounds it, per pair in FP32 (HBM at 6.8 TB/s, the FMA pipe, shared memory at
+// 128 bytes a cycle and SM; measured): plane 96^3 2.1, 6.1, 6.8; 9.9 us (start: 8.2
+// for z alone, 17.5 with the y passes of the slab kernels), 160^3 9.7, 34, 32; 59 us.
+// xfwd 96^3 1.0 us of HBM, 1.9 measured; 160^3 4.9 and 9.0 (exchange through shared
+// memory 60% busy).  xinv 96^3 1.6 and 1.9; 160^3 7.3 and 8.2.
 #pragma once
 
 #include <cstring>
@@ -145,6 +151,13 @@ template <int H, typename C> __device__ __forceinline__ void stash_get(unsigned 
 }
 
 // -------------------------------------------------------------------- plane
+// Shared memory, the FMA pipe and instruction issue are each about 65% busy; HBM
+// 20%.  Hence: every pass in place (the plane is all the shared memory there
+// is), odd pitch and lanes across lines (no bank conflicts, warp-uniform
+// twiddles read two at a time), barriers of groups rather than of the CTA, and
+// the z samples and partial outputs in tensor memory rather than a second half
+// of every z spectrum in shared memory.
+//
 // Launch shape and on-chip layout of the plane kernel for grids of G points,
 // (y, z) lines periodic or free.  The plane P[row][z] holds the y spectrum
 // (row = ky in natural order) of the G z-samples, row pitch ZP odd, so that
