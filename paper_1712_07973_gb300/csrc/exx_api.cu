@@ -286,7 +286,8 @@ struct exx_plan_s {
   void* Gs = nullptr;
   void* tw = nullptr;
   void* twz = nullptr;  // twiddles of the z transform where its length differs
-  double* d_occ = nullptr;
+  double* d_occ = nullptr;  // occupations, then the gradient's factors -alpha 2 h^3 f_k
+  float* d_occf = nullptr;  // behind them: the occupations in FP32
   int4* d_pairs = nullptr;
   double* epart = nullptr;
   double* Epair = nullptr;
@@ -418,18 +419,18 @@ int default_tile(int N, int requested) {
 constexpr unsigned kWideBlocks = 400;
 // k_accum launch: vector width 2 when aligned, full-tile specialisations
 template <typename R, int VEC>
-void launch_accum_v(int mode, const R* psi, const R* V, double* acc, const double* occ,
-                    const Tile& t, double c, double gs, long long n3, int touch, R* out, cudaStream_t st) {
+void launch_accum_v(int mode, const R* psi, const R* V, double* acc, const R* occ, const double* coef,
+                    const Tile& t, double c, long long n3, int touch, R* out, cudaStream_t st) {
   const int threads = kAccumThreads;
   const unsigned blocks = (unsigned)((n3 / VEC + threads - 1) / threads);
   if (blocks < kWideBlocks) {
     const dim3 grid(blocks, t.diag ? t.ti : t.ti + t.tj);
-    launch_dep(k_accum_wide<R, 8, VEC>, grid, threads, 0, st, psi, V, acc, occ, t.i0, t.ti, t.j0, t.tj, t.diag, c,
-               gs, n3, touch, out);
+    launch_dep(k_accum_wide<R, 8, VEC>, grid, threads, 0, st, psi, V, acc, occ, coef, t.i0, t.ti, t.j0, t.tj,
+               t.diag, c, n3, touch, out);
     return;
   }
   auto go = [&](auto k) {
-    launch_dep(k, dim3(blocks), threads, 0, st, psi, V, acc, occ, t.i0, t.ti, t.j0, t.tj, t.diag, c, gs, n3, touch,
+    launch_dep(k, dim3(blocks), threads, 0, st, psi, V, acc, occ, coef, t.i0, t.ti, t.j0, t.tj, t.diag, c, n3, touch,
                out);
   };
   auto by_mode = [&](auto T) {
@@ -450,16 +451,16 @@ void launch_accum_v(int mode, const R* psi, const R* V, double* acc, const doubl
   by_mode(ic<-1>{});
 }
 template <typename R>
-void launch_accum(bool v2, int mode, const R* psi, const R* V, double* acc, const double* occ,
-                  const Tile& t, double c, double gs, long long n3, int touch, R* out, cudaStream_t st) {
+void launch_accum(bool v2, int mode, const R* psi, const R* V, double* acc, const R* occ, const double* coef,
+                  const Tile& t, double c, long long n3, int touch, R* out, cudaStream_t st) {
   if constexpr (sizeof(R) == 4) {  // four FP32 values per thread: -4% at 160^3
     if (v2 && (n3 % 4) == 0) {
-      launch_accum_v<R, 4>(mode, psi, V, acc, occ, t, c, gs, n3, touch, out, st);
+      launch_accum_v<R, 4>(mode, psi, V, acc, occ, coef, t, c, n3, touch, out, st);
       return;
     }
   }
-  if (v2) launch_accum_v<R, 2>(mode, psi, V, acc, occ, t, c, gs, n3, touch, out, st);
-  else launch_accum_v<R, 1>(mode, psi, V, acc, occ, t, c, gs, n3, touch, out, st);
+  if (v2) launch_accum_v<R, 2>(mode, psi, V, acc, occ, coef, t, c, n3, touch, out, st);
+  else launch_accum_v<R, 1>(mode, psi, V, acc, occ, coef, t, c, n3, touch, out, st);
 }
 
 extern "C" {
@@ -645,7 +646,8 @@ static exx_status_t plan_create_impl(exx_plan_t* out, const int grid[3], const d
   if (!twzbuf.empty()) {
     EXX_ALLOC(p->twz, twzbuf.size());
   }
-  EXX_ALLOC(p->d_occ, norb * sizeof(double));
+  EXX_ALLOC(p->d_occ, norb * (2 * sizeof(double) + sizeof(float)));
+  p->d_occf = reinterpret_cast<float*>(p->d_occ + 2 * (size_t)norb);
   EXX_ALLOC(p->d_pairs, pairs.size() * sizeof(int4));
   EXX_ALLOC(p->epart, (size_t)p->maxpairs * nper * sizeof(double));
   EXX_ALLOC(p->Epair, (size_t)p->P * sizeof(double));
@@ -675,12 +677,19 @@ static exx_status_t plan_create_impl(exx_plan_t* out, const int grid[3], const d
   }
 #undef EXX_ALLOC
 
+  std::vector<double> occbuf(2 * (size_t)norb + ((size_t)norb + 1) / 2);
+  const double gs = 2.0 * (p->h * p->h * p->h);
+  for (int k = 0; k < norb; ++k) {
+    occbuf[k] = p->occ[k];
+    occbuf[norb + k] = -p->alpha * (gs * p->occ[k]);
+    reinterpret_cast<float*>(occbuf.data() + 2 * (size_t)norb)[k] = (float)p->occ[k];
+  }
   cudaError_t e = cudaMemcpyAsync(p->Gs, gbuf.data(), gbuf.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(p->tw, twbuf.data(), twbuf.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && p->twz)
     e = cudaMemcpyAsync(p->twz, twzbuf.data(), twzbuf.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(p->d_occ, p->occ.data(), norb * sizeof(double), cudaMemcpyHostToDevice, st);
+    e = cudaMemcpyAsync(p->d_occ, occbuf.data(), norb * (2 * sizeof(double) + sizeof(float)), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(p->d_pairs, pairs.data(), pairs.size() * sizeof(int4), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(p->Epair, 0, (size_t)p->P * sizeof(double), st);
@@ -767,7 +776,7 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
     if (p->sharded) EXX_CUDA(p, cudaMemsetAsync(acc, 0, (size_t)N * n3 * sizeof(double), st));
   }
   const double c = -p->alpha;
-  const double gs = grad ? 2.0 * h3 : 0.0;
+  const double* coef = grad ? p->d_occ + N : nullptr;  // gradient: factor of each orbital
   if (p->sharded)  // pair energies of other ranks' tiles must read as zero
     EXX_CUDA(p, cudaMemsetAsync(p->Epair, 0, (size_t)p->P * sizeof(double), st));
   // Lanes: consecutive tiles go round-robin over the lanes' streams, each with
@@ -861,10 +870,10 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
         ProfScope ps(p, K_ACCUM, st);
         if (p->prec == EXX_FP64)
           launch_accum<double>(v2, mode, static_cast<const double*>(psi), static_cast<const double*>(Vt), acc,
-                               p->d_occ, t, c, gs, n3, touch, nullptr, st);
+                               p->d_occ, coef, t, c, n3, touch, nullptr, st);
         else
           launch_accum<float>(v2, mode, static_cast<const float*>(psi), static_cast<const float*>(Vt), acc,
-                              p->d_occ, t, c, gs, n3, touch, out, st);
+                              p->d_occf, coef, t, c, n3, touch, out, st);
       }
       if (nl > 1) EXX_CUDA(p, cudaEventRecord(p->ev_free[l], st));
       if (ov && row_end) EXX_CUDA(p, cudaEventRecord((*ov->out)[t.i0 / p->T], st));

@@ -131,7 +131,9 @@ struct exx_batch_s {
   // device
   int4* d_pairs = nullptr;
   TileDesc* d_tiles = nullptr;
-  double* d_occ = nullptr;
+  double* d_occ = nullptr;   // occupations of all molecules' orbitals, the gradient's factors
+  double* d_coef = nullptr;  // -alpha 2 h^3 f_k behind them, then the occupations in FP32
+  float* d_occf = nullptr;
   double* Epair = nullptr;
   double* epart = nullptr;
   int* d_err = nullptr;  // set by a device-side wait that ran out
@@ -326,13 +328,13 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
       a.tw = static_cast<const float2*>(g.plane ? g.tw_q : g.tw);
       a.Epair = b->Epair;
       a.vx_tab = b->d_vacc_tab;
-      a.occ = b->d_occ;
+      a.occ = b->d_occf;
+      a.coef = grad ? b->d_coef : nullptr;
       a.qc = b->d_qc;
       a.err = b->d_err;
       a.h3 = g.h * g.h * g.h;
       a.n3 = n3;
       a.nblk = g.nblk;
-      a.grad = grad ? 1 : 0;
       a.energy_only = apply ? 0 : 1;
       a.vec2 = (b->vec2 && (n3 % 2) == 0) ? 1 : 0;
       if (g.ops->persist(a, st) != cudaSuccess) return EXX_ERR_CUDA;
@@ -375,8 +377,8 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
         launch_dep(vec == 4   ? k_accum_batch<float, 8, 4>
                    : vec == 2 ? k_accum_batch<float, 8, 2>
                               : k_accum_batch<float, 8, 1>,
-                   dim3((unsigned)blocks, w.ntile), threads, 0, st, b->d_psi_tab, static_cast<const float*>(Vl[l]), b->d_vacc_tab, out, b->d_occ,
-                   b->d_tiles + w.tile_off, grad ? 1 : 0, n3);
+                   dim3((unsigned)blocks, w.ntile), threads, 0, st, b->d_psi_tab, static_cast<const float*>(Vl[l]), b->d_vacc_tab, out, b->d_occf,
+                   grad ? b->d_coef : nullptr, b->d_tiles + w.tile_off, n3);
         if (nl > 1 && cudaEventRecord(b->ev_free[l], st) != cudaSuccess) return EXX_ERR_CUDA;
       }
     }
@@ -547,7 +549,6 @@ exx_status_t exx_batch_create(exx_batch_t* out, int nmol, const exx_mol_desc* mo
           t.mol = g.mols[k];
           t.occ_off = m.occ_off;
           t.c = -m.alpha;
-          t.g2h3 = 2.0 * m.h * m.h * m.h;
           t.voff = 0;
           t.touch = (bi == 0 ? (t.diag ? T_FIRST_I : T_FIRST_J) : 0) | (bj == nb - 1 ? T_LAST_I : 0);
           std::vector<int4> ps;
@@ -600,7 +601,7 @@ exx_status_t exx_batch_create(exx_batch_t* out, int nmol, const exx_mol_desc* mo
   }
   bool ok = balloc(b, &b->d_pairs, b->pairs.size() * sizeof(int4)) &&
             balloc(b, &b->d_tiles, b->tiles.size() * sizeof(TileDesc)) &&
-            balloc(b, &b->d_occ, occ.size() * sizeof(double)) &&
+            balloc(b, &b->d_occ, occ.size() * (2 * sizeof(double) + sizeof(float))) &&
             balloc(b, &b->Epair, (size_t)ep * sizeof(double)) && balloc(b, &b->epart, b->ep_bytes) &&
             balloc(b, &b->X, b->x_bytes) && balloc(b, &b->V, b->v_bytes) &&
             balloc(b, &b->vacc, (size_t)vo * sizeof(double)) &&
@@ -622,7 +623,15 @@ exx_status_t exx_batch_create(exx_batch_t* out, int nmol, const exx_mol_desc* mo
   };
   up(b->d_pairs, b->pairs.data(), b->pairs.size() * sizeof(int4));
   up(b->d_tiles, b->tiles.data(), b->tiles.size() * sizeof(TileDesc));
+  std::vector<double> coef(occ.size());
+  for (const Mol& m : b->mol)
+    for (int k = 0; k < m.N; ++k) coef[m.occ_off + k] = -m.alpha * ((2.0 * m.h * m.h * m.h) * occ[m.occ_off + k]);
+  const std::vector<float> occf(occ.begin(), occ.end());
+  b->d_coef = b->d_occ + occ.size();
+  b->d_occf = reinterpret_cast<float*>(b->d_coef + occ.size());
   up(b->d_occ, occ.data(), occ.size() * sizeof(double));
+  up(b->d_coef, coef.data(), coef.size() * sizeof(double));
+  up(b->d_occf, occf.data(), occf.size() * sizeof(float));
   up(b->d_mt, mt.data(), mt.size() * sizeof(MolTot));
   up(b->d_vacc_tab, vtab.data(), vtab.size() * sizeof(double*));
   up(b->d_count, count.data(), count.size() * sizeof(long long));

@@ -900,6 +900,16 @@ __device__ __forceinline__ void vstream(const R* p, R (&v)[VEC]) {
     for (int e = 0; e < VEC; ++e) v[e] = q[e];
   }
 }
+// (double)x for the FP64 accumulation.  GB300 converts on its FP64 units, two
+// values per cycle and SM; a normal number's bits move over with integer
+// instructions instead (exact: the mantissa widens, the exponent's bias grows by
+// 896).
+__device__ __forceinline__ double to_f64(double x) { return x; }
+__device__ __forceinline__ double to_f64(float x) {
+  const unsigned u = __float_as_uint(x), e = u & 0x7f800000u;
+  if (e == 0u || e == 0x7f800000u) return (double)x;  // zero, subnormal, infinite, NaN
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
 // vx[0..VEC) += c * a  (FP64); first: the accumulator counts as zero and is
 // not read; out != null: the sum goes there in the working precision (the
 // orbital's last update), not back to the accumulator.  The same sums, bit for
@@ -920,7 +930,7 @@ __device__ __forceinline__ void vacc(double* p, double c, const R (&a)[VEC], boo
     }
   }
 #pragma unroll
-  for (int e = 0; e < VEC; ++e) u[e] += c * (double)a[e];
+  for (int e = 0; e < VEC; ++e) u[e] += c * to_f64(a[e]);
   if (out != nullptr) {
     if constexpr (sizeof(R) == 4 && VEC == 4) {
       *reinterpret_cast<float4*>(out) = make_float4((float)u[0], (float)u[1], (float)u[2], (float)u[3]);
@@ -946,21 +956,23 @@ enum Touch { T_FIRST_I = 1, T_FIRST_J = 2, T_LAST_I = 4 };
 // compile-time constant, so that all loads of a J step can be issued at once
 // (with the register budget of two CTAs per SM: 4.9 -> 3.8 ms per exx_apply
 // at n = 96, 64 orbitals).
-// gs = 0: the exchange action, vx_k += c * sum; gs > 0: the gradient of E_x,
-// vx_k += c gs f_k * sum (gs = 2 h^3: dE_x/dpsi_k = 2 f_k h^3 (Vx psi)_k,
-// Eq. daction), the per-orbital factor folded into the FP64 accumulation.
+// coef = null: the exchange action, vx_k += c * sum; else the gradient of E_x,
+// vx_k += coef_k * sum, coef_k = -alpha 2 h^3 f_k (dE_x/dpsi_k = 2 f_k h^3 (Vx
+// psi)_k, Eq. daction), the per-orbital factor folded into the FP64
+// accumulation.  occ: the occupations in the working precision.  (Forming both
+// per thread, and converting the sums on the FP64 units, kept those 66% busy.)
 // touch: Touch bits; out: the output that takes an orbital's last update.
 template <typename R, int TM, int VEC, int MODE, bool COH = false>
 __device__ __forceinline__ void accum_tile(const R* __restrict__ psi, const R* __restrict__ V,
-                                           double* __restrict__ vx,
-                                           const double* __restrict__ occ, int i0, int ti_,
-                                           int j0, int tj_, int diag_, double c, double gs,
+                                           double* __restrict__ vx, const R* __restrict__ occ,
+                                           const double* __restrict__ coef, int i0, int ti_,
+                                           int j0, int tj_, int diag_, double c,
                                            long long n3, long long r, int touch, R* out) {
   const int ti = MODE ? TM : ti_, tj = MODE ? TM : tj_;
   const bool diag = MODE == 2 ? true : MODE == 1 ? false : diag_ != 0;
   R fi[TM];
 #pragma unroll
-  for (int a = 0; a < TM; ++a) fi[a] = a < ti ? (R)occ[i0 + a] : R(0);
+  for (int a = 0; a < TM; ++a) fi[a] = a < ti ? occ[i0 + a] : R(0);
   R pi[TM][VEC], ai[TM][VEC];
 #pragma unroll
   for (int a = 0; a < TM; ++a) {
@@ -971,7 +983,7 @@ __device__ __forceinline__ void accum_tile(const R* __restrict__ psi, const R* _
 #pragma unroll
   for (int b = 0; b < TM; ++b) {
     if (b >= tj) break;
-    const R fb = (R)occ[j0 + b];
+    const R fb = occ[j0 + b];
     R pb[VEC], aj[VEC];
     if (diag) {
 #pragma unroll
@@ -998,14 +1010,14 @@ __device__ __forceinline__ void accum_tile(const R* __restrict__ psi, const R* _
 #pragma unroll
       for (int e = 0; e < VEC; ++e) ai[b][e] += aj[e];
     } else {
-      const double cb = gs != 0.0 ? c * (gs * occ[j0 + b]) : c;
+      const double cb = coef ? coef[j0 + b] : c;
       vacc<R, VEC, COH>(vx + (long long)(j0 + b) * n3 + r, cb, aj, (touch & T_FIRST_J) != 0, nullptr);
     }
   }
 #pragma unroll
   for (int a = 0; a < TM; ++a)
     if (a < ti) {
-      const double ca = gs != 0.0 ? c * (gs * occ[i0 + a]) : c;
+      const double ca = coef ? coef[i0 + a] : c;
       const long long o = (long long)(i0 + a) * n3 + r;
       vacc<R, VEC, COH>(vx + o, ca, ai[a], (touch & T_FIRST_I) != 0, out != nullptr ? out + o : nullptr);
     }
@@ -1021,12 +1033,12 @@ constexpr int kAccumThreads = 128;
 template <typename R, int TM, int VEC, int MODE, int TOUCH>
 __global__ void __launch_bounds__(kAccumThreads, (sizeof(R) == 4 && MODE == 0) ? 6 : 4)
 k_accum(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__ vx,
-        const double* __restrict__ occ, int i0, int ti, int j0, int tj, int diag, double c,
-        double gs, long long n3, int touch, R* out) {
+        const R* __restrict__ occ, const double* __restrict__ coef, int i0, int ti, int j0, int tj, int diag,
+        double c, long long n3, int touch, R* out) {
   dep_wait();
   const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * VEC;
   if (r >= n3) return;
-  accum_tile<R, TM, VEC, MODE>(psi, V, vx, occ, i0, ti, j0, tj, diag, c, gs, n3, r,
+  accum_tile<R, TM, VEC, MODE>(psi, V, vx, occ, coef, i0, ti, j0, tj, diag, c, n3, r,
                                TOUCH < 0 ? touch : TOUCH, TOUCH < 0 || (TOUCH & T_LAST_I) ? out : nullptr);
 }
 
@@ -1037,8 +1049,8 @@ k_accum(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__
 template <typename R, int TM, int VEC>
 __global__ void __launch_bounds__(kAccumThreads)
 k_accum_wide(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__ vx,
-             const double* __restrict__ occ, int i0, int ti, int j0, int tj, int diag, double c,
-             double gs, long long n3, int touch, R* out) {
+             const R* __restrict__ occ, const double* __restrict__ coef, int i0, int ti, int j0, int tj, int diag,
+             double c, long long n3, int touch, R* out) {
   dep_wait();
   const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * VEC;
   if (r >= n3) return;
@@ -1057,7 +1069,7 @@ k_accum_wide(const R* __restrict__ psi, const R* __restrict__ V, double* __restr
       const int slot = diag ? a * tj - (a * (a - 1)) / 2 + (b - a) : a * tj + b;
       vload<R, VEC>(V + (long long)slot * n3 + r, v[m]);
       vload<R, VEC>(psi + (long long)(o0 + m) * n3 + r, q[m]);
-      f[m] = (R)occ[o0 + m];
+      f[m] = occ[o0 + m];
     }
   }
   R acc[VEC];
@@ -1093,7 +1105,7 @@ k_accum_wide(const R* __restrict__ psi, const R* __restrict__ V, double* __restr
     }
   }
   const int ko = (on_i ? i0 : j0) + k;
-  const double ck = gs != 0.0 ? c * (gs * occ[ko]) : c;
+  const double ck = coef ? coef[ko] : c;
   const long long o = (long long)ko * n3 + r;
   vacc<R, VEC>(vx + o, ck, acc, (touch & (on_i ? T_FIRST_I : T_FIRST_J)) != 0,
                on_i && out != nullptr ? out + o : nullptr);
@@ -1107,12 +1119,11 @@ struct TileDesc {
   int mol;    // molecule slot: psi_tab[mol], vx_tab[mol], occ + occ_off[mol]
   int occ_off;
   double c;   // -alpha of the molecule
-  double g2h3;  // 2 h^3 of the molecule (gradient calls)
   int touch;    // Touch bits
 };
 
 // One tile per blockIdx.y; full tiles take the specialised bodies (the branch
-// is uniform over a block).  grad != 0: gradient of E_x (see accum_tile).
+// is uniform over a block).  coef: as in accum_tile (all molecules' orbitals).
 // vx_out (table of output arrays): the tiles' Touch bits count; null: they do
 // not (the accumulators are cleared and converted in passes of their own).
 template <typename R, int TM, int VEC, bool COH>
@@ -1120,8 +1131,9 @@ __device__ __forceinline__ void accum_batch_unit(const R* const* __restrict__ ps
                                                  const R* __restrict__ V,
                                                  double* const* __restrict__ vx_tab,
                                                  R* const* __restrict__ vx_out,
-                                                 const double* __restrict__ occ,
-                                                 const TileDesc* __restrict__ tiles, int grad,
+                                                 const R* __restrict__ occ,
+                                                 const double* __restrict__ coef,
+                                                 const TileDesc* __restrict__ tiles,
                                                  long long n3, const int bx, const int by,
                                                  const int nt) {
   const TileDesc t = tiles[by];
@@ -1129,18 +1141,18 @@ __device__ __forceinline__ void accum_batch_unit(const R* const* __restrict__ ps
   if (r >= n3) return;
   const R* __restrict__ psi = psi_tab[t.mol];
   double* __restrict__ vx = vx_tab[t.mol];
-  const double* __restrict__ oc = occ + t.occ_off;
+  const R* __restrict__ oc = occ + t.occ_off;
+  const double* __restrict__ cf = coef ? coef + t.occ_off : nullptr;
   const R* __restrict__ Vt = V + (long long)t.voff * n3;
-  const double gs = grad ? t.g2h3 : 0.0;
   const int touch = vx_out ? t.touch : 0;
   R* out = (touch & T_LAST_I) ? vx_out[t.mol] : nullptr;
   if (t.ti == TM && t.tj == TM) {
     if (t.diag)
-      accum_tile<R, TM, VEC, 2, COH>(psi, Vt, vx, oc, t.i0, TM, t.j0, TM, 1, t.c, gs, n3, r, touch, out);
+      accum_tile<R, TM, VEC, 2, COH>(psi, Vt, vx, oc, cf, t.i0, TM, t.j0, TM, 1, t.c, n3, r, touch, out);
     else
-      accum_tile<R, TM, VEC, 1, COH>(psi, Vt, vx, oc, t.i0, TM, t.j0, TM, 0, t.c, gs, n3, r, touch, out);
+      accum_tile<R, TM, VEC, 1, COH>(psi, Vt, vx, oc, cf, t.i0, TM, t.j0, TM, 0, t.c, n3, r, touch, out);
   } else {
-    accum_tile<R, TM, VEC, 0, COH>(psi, Vt, vx, oc, t.i0, t.ti, t.j0, t.tj, t.diag, t.c, gs, n3, r, touch, out);
+    accum_tile<R, TM, VEC, 0, COH>(psi, Vt, vx, oc, cf, t.i0, t.ti, t.j0, t.tj, t.diag, t.c, n3, r, touch, out);
   }
 }
 
@@ -1148,9 +1160,10 @@ template <typename R, int TM, int VEC>
 __global__ void __launch_bounds__(kAccumThreads, 4)
 k_accum_batch(const R* const* __restrict__ psi_tab, const R* __restrict__ V,
               double* const* __restrict__ vx_tab, R* const* __restrict__ vx_out,
-              const double* __restrict__ occ, const TileDesc* __restrict__ tiles, int grad, long long n3) {
+              const R* __restrict__ occ, const double* __restrict__ coef, const TileDesc* __restrict__ tiles,
+              long long n3) {
   dep_wait();
-  accum_batch_unit<R, TM, VEC, false>(psi_tab, V, vx_tab, vx_out, occ, tiles, grad, n3, blockIdx.x,
+  accum_batch_unit<R, TM, VEC, false>(psi_tab, V, vx_tab, vx_out, occ, coef, tiles, n3, blockIdx.x,
                                       blockIdx.y, blockDim.x);
 }
 

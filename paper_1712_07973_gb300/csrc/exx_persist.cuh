@@ -59,13 +59,14 @@ struct PersistArgs {
   const float2* tw;             // twiddles of the group
   double* Epair;
   double* const* vx_tab;        // FP64 accumulators per molecule slot
-  const double* occ;
+  const float* occ;             // occupations, and the gradient's factors (null: the action)
+  const double* coef;
   int* qc;                      // [0] queue head, [1..nseg] done counts, [nseg+1] abort
   int* err;                     // [0] set when a wait ran out
   double h3;
   long long n3;
   int nblk;                     // accumulation point blocks per tile
-  int grad, energy_only, vec2;
+  int energy_only, vec2;
 };
 
 constexpr int kQueuePolls = 1 << 20;  // bound of every queue wait (x ~0.25-1 us per poll)
@@ -164,11 +165,11 @@ __global__ void __launch_bounds__(NT, MINB) k_persist(const PersistArgs a) {
       } else {
         const int t = u / a.nblk, b = u - t * a.nblk;
         if (a.vec2)
-          accum_batch_unit<float, 8, 2, true>(a.psi_tab, a.V[sg.slot], a.vx_tab, nullptr, a.occ,
-                                              a.tiles + sg.tile_off, a.grad, a.n3, b, t, NT);
+          accum_batch_unit<float, 8, 2, true>(a.psi_tab, a.V[sg.slot], a.vx_tab, nullptr, a.occ, a.coef,
+                                              a.tiles + sg.tile_off, a.n3, b, t, NT);
         else
-          accum_batch_unit<float, 8, 1, true>(a.psi_tab, a.V[sg.slot], a.vx_tab, nullptr, a.occ,
-                                              a.tiles + sg.tile_off, a.grad, a.n3, b, t, NT);
+          accum_batch_unit<float, 8, 1, true>(a.psi_tab, a.V[sg.slot], a.vx_tab, nullptr, a.occ, a.coef,
+                                              a.tiles + sg.tile_off, a.n3, b, t, NT);
       }
     }
     __syncthreads();  // then one release by thread 0 publishes the whole CTA's results
