@@ -151,6 +151,9 @@ exx_status_t exx_energy(exx_plan_t plan, const void* psi, double* E_out, void* c
  *   psi    device, as for exx_energy.
  *   vxpsi  device, [norb][n][n][n]; double for EXX_FP64 or with
  *          EXX_FLAG_VX_FP64, else float.  Overwritten (not accumulated).
+ *          A float vxpsi may share memory with psi (in-place calls, shifted
+ *          views); a double one, in which the sums themselves are held, must
+ *          not.
  *   E_out  host, may be NULL.  If non-NULL the call synchronises the stream.
  * The gradient of E_x is dE_x/dpsi_k = 2 f_k h^3 (Vx psi)_k.
  */
@@ -321,7 +324,8 @@ exx_status_t exx_batch_create(exx_batch_t* out, int nmol, const exx_mol_desc* mo
  * host arrays of nmol device pointers (float [norb_m][n_m]^3 each); vxpsi may
  * be NULL for energy-only use.  The pointers are copied into device tables
  * that later calls (and captured graphs) read, so rebinding does not require
- * a new capture.  Synchronises the stream.
+ * a new capture.  Outputs may share memory with orbitals, of the same or of
+ * other molecules.  Synchronises the stream.
  */
 exx_status_t exx_batch_set_buffers(exx_batch_t batch, const float* const* psi,
                                    float* const* vxpsi, void* cuda_stream);

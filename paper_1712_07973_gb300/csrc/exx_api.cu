@@ -759,6 +759,12 @@ struct HostOverlap {
   const std::vector<cudaEvent_t>* out;
 };
 
+// Do the orbitals and the output share memory?
+static bool buffers_overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
+  return pa < pb + nb && pb < pa + na;
+}
+
 // apply: also the inverse transforms and the accumulation into vxpsi, which
 // receives (Vx psi)_k (grad = false) or dE_x/dpsi_k = 2 f_k h^3 (Vx psi)_k
 // (grad = true).
@@ -769,9 +775,14 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
   const double h3 = p->h * p->h * p->h;
   const int nper = p->nper;
   double* acc = nullptr;
+  // FP32 output converted by a pass of its own behind all tiles, not by each
+  // orbital's last update: a shard's tiles need not hold that update, and an
+  // output that shares memory with the orbitals (an in-place call) must not be
+  // written while tiles, or other CTAs of the same one, still read them
+  const size_t out_bytes = (size_t)N * n3 * sizeof(float);
+  const bool convert = apply && p->vacc && (p->sharded || buffers_overlap(psi, out_bytes, vxpsi, out_bytes));
   if (apply) {
-    // every orbital's first update clears and (FP32 output) its last converts,
-    // where this plan runs all tiles; a shard's tiles need not hold either
+    // every orbital's first update clears, where this plan runs all tiles
     acc = p->vacc ? p->vacc : static_cast<double*>(vxpsi);
     if (p->sharded) EXX_CUDA(p, cudaMemsetAsync(acc, 0, (size_t)N * n3 * sizeof(double), st));
   }
@@ -847,7 +858,7 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
       int touch = 0;
       if (!p->sharded) {
         if (t.i0 == 0) touch = t.diag ? T_FIRST_I : T_FIRST_J;
-        if (row_end && p->vacc) touch |= T_LAST_I;  // (no conversion of an FP64 output)
+        if (row_end && p->vacc && !convert) touch |= T_LAST_I;  // (no conversion of an FP64 output)
       }
       float* out = (touch & T_LAST_I) ? static_cast<float*>(vxpsi) : nullptr;
       const bool al = ((uintptr_t)psi % 16 == 0) && ((uintptr_t)acc % 16 == 0) &&
@@ -888,7 +899,7 @@ static exx_status_t run(exx_plan_t p, const void* psi, void* vxpsi, double* E_de
     ProfScope ps(p, K_TOTAL, st);
     launch_dep(k_exx_total, dim3(1), 256, 0, st, p->Epair, p->P, N, p->d_occ, p->alpha, E_dev ? E_dev : p->E_dev);
   }
-  if (apply && p->vacc && p->sharded) {
+  if (convert) {
     ProfScope ps(p, K_CONV, st);
     const long long tot = (long long)N * n3;
     long long blocks = (tot + 255) / 256;

@@ -147,6 +147,7 @@ struct exx_batch_s {
   long long* d_count = nullptr;
   bool have_vx = false;
   bool buffers_set = false;
+  bool aliased = false;  // an output shares memory with orbitals (in-place calls): converted behind all waves
   bool vec4 = true;  // every orbital and output array 16-byte aligned: loads and stores of four
   bool vec2 = true;  // every orbital array 8-byte aligned: paired loads in accum
   // second pipeline lane (as in a single plan): its workspaces, streams, events
@@ -284,8 +285,10 @@ void build_segments(exx_batch_t b, Group& g, bool apply, bool stall, std::vector
 
 exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaStream_t st) {
   // launch per pass: every orbital's first update clears and its last converts
-  // (TileDesc::touch); the persistent queue clears and converts in passes
-  if (apply && b->persistent) {
+  // (TileDesc::touch); the persistent queue, and outputs that must not be
+  // written before the last read of the orbitals, clear and convert in passes
+  const bool passes = b->persistent || b->aliased;
+  if (apply && passes) {
     const Mol& last = b->mol.back();
     const long long tot = last.vacc_off + (long long)last.N * last.n * last.n * last.n;
     if (cudaMemsetAsync(b->vacc, 0, (size_t)tot * sizeof(double), st) != cudaSuccess) return EXX_ERR_CUDA;
@@ -370,7 +373,7 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
           return EXX_ERR_CUDA;
         used[l] = true;
         energies();
-        float* const* out = b->persistent ? nullptr : b->d_vx_tab;
+        float* const* out = passes ? nullptr : b->d_vx_tab;
         const int vec = b->vec4 && (n3 % 4) == 0 ? 4 : b->vec2 && (n3 % 2) == 0 ? 2 : 1;
         const int threads = kAccumThreads;
         const long long blocks = (n3 / vec + threads - 1) / threads;
@@ -389,7 +392,7 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
           cudaStreamWaitEvent(st, b->ev_done[l], 0) != cudaSuccess)
         return EXX_ERR_CUDA;
   k_exx_total_batch<<<b->nmol, 256, 0, st>>>(b->Epair, b->d_mt, b->d_occ, E_dev);
-  if (apply && b->have_vx && b->persistent) {
+  if (apply && b->have_vx && passes) {
     long long mx = 0;
     for (const Mol& m : b->mol) mx = std::max(mx, (long long)m.N * m.n * m.n * m.n);
     const long long blocks = std::min<long long>((mx + 255) / 256, 1024);
@@ -397,6 +400,25 @@ exx_status_t enqueue(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaSt
                                                                        b->d_count);
   }
   return cudaGetLastError() == cudaSuccess ? EXX_OK : EXX_ERR_CUDA;
+}
+
+// Does any molecule's output share memory with any molecule's orbitals?
+bool buffers_overlap(exx_batch_t b, const std::vector<const float*>& psi, const std::vector<float*>& vx) {
+  std::vector<std::pair<uintptr_t, uintptr_t>> in;  // [begin, end) of the orbitals by begin,
+  for (int m = 0; m < b->nmol; ++m) {
+    const Mol& d = b->mol[m];
+    const uintptr_t a = reinterpret_cast<uintptr_t>(psi[m]);
+    in.emplace_back(a, a + (size_t)d.N * d.n * d.n * d.n * sizeof(float));
+  }
+  std::sort(in.begin(), in.end());
+  for (size_t k = 1; k < in.size(); ++k) in[k].second = std::max(in[k].second, in[k - 1].second);  // furthest end so far
+  for (int m = 0; m < b->nmol; ++m) {
+    const Mol& d = b->mol[m];
+    const uintptr_t a = reinterpret_cast<uintptr_t>(vx[m]), e = a + (size_t)d.N * d.n * d.n * d.n * sizeof(float);
+    const auto it = std::lower_bound(in.begin(), in.end(), std::make_pair(e, (uintptr_t)0));  // begins at e or later
+    if (it != in.begin() && (it - 1)->second > a) return true;
+  }
+  return false;
 }
 
 exx_status_t run_batch(exx_batch_t b, double* E_dev, bool apply, bool grad, cudaStream_t st) {
@@ -714,7 +736,8 @@ exx_status_t exx_batch_set_buffers(exx_batch_t b, const float* const* psi, float
     v2 = v2 && ((uintptr_t)p[m] % 8 == 0);
     v4 = v4 && ((uintptr_t)p[m] % 16 == 0) && ((uintptr_t)v[m] % 16 == 0);
   }
-  if (v2 != b->vec2 || v4 != b->vec4 || have != b->have_vx) {  // the captured graphs embed these choices
+  const bool al = have && buffers_overlap(b, p, v);
+  if (v2 != b->vec2 || v4 != b->vec4 || have != b->have_vx || al != b->aliased) {  // the captured graphs embed these choices
     for (int k = 0; k < 3; ++k)
       if (b->gexec[k]) {
         cudaGraphExecDestroy(b->gexec[k]);
@@ -723,6 +746,7 @@ exx_status_t exx_batch_set_buffers(exx_batch_t b, const float* const* psi, float
   }
   b->vec2 = v2;
   b->vec4 = v4;
+  b->aliased = al;
   b->have_vx = have;
   b->buffers_set = true;
   return EXX_OK;
@@ -861,7 +885,7 @@ exx_status_t exx_batch_info(exx_batch_t b, int* ngroups, int* nwaves, size_t* wo
   if (nwaves) *nwaves = nw;
   if (workspace_bytes) *workspace_bytes = b->ws;
   if (launches_apply) {
-    int la = b->persistent ? 2 : 1;  // E_x totals (and the conversion of the outputs)
+    int la = b->persistent || b->aliased ? 2 : 1;  // E_x totals (and the conversion of the outputs)
     for (const Group& g : b->groups)
       la += (b->persistent && g.ops->persist_ok) ? 1 : 5 * (int)g.waves.size();
     *launches_apply = la;
