@@ -17,6 +17,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstdlib>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -126,6 +127,7 @@ struct exx_batch_s {
   std::vector<int4> pairs;
   std::vector<TileDesc> tiles;
   size_t ws = 0;
+  int fail_alloc = 0, nalloc = 0;  // test hook: this allocation (1-based) of an enable reports out of memory
   int max_wave_pairs = 0;
   size_t x_bytes = 0, v_bytes = 0, ep_bytes = 0;
   // device
@@ -200,6 +202,7 @@ void batch_free(exx_batch_t b) {
 
 template <typename T> bool balloc(exx_batch_t b, T** p, size_t bytes) {
   void* q = nullptr;
+  if (b->fail_alloc > 0 && ++b->nalloc == b->fail_alloc) return false;
   if (cudaMalloc(&q, bytes ? bytes : 16) != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -459,6 +462,7 @@ exx_status_t run_batch(exx_batch_t b, double* E_dev, bool apply, bool grad, cuda
 
 // Kernel table and twiddles of a group, built on the host and copied (plane:
 // the plane pipeline's layout, else the slab pipeline's); synchronises st.
+// Both or, on failure, neither.
 exx_status_t group_tables(exx_batch_t b, const Group& g, bool plane, void** Gs, void** tw, cudaStream_t st) {
   const Ops* ops = g.ops;
   const size_t m = (size_t)g.n + 1;
@@ -478,13 +482,96 @@ exx_status_t group_tables(exx_batch_t b, const Group& g, bool plane, void** Gs, 
                                    gf.data());
     exx::build_twiddles(g.n, twf.data());
   }
-  if (!balloc(b, Gs, gf.size()) || !balloc(b, tw, twf.size() * sizeof(float))) return EXX_ERR_OOM;
+  const size_t ws = b->ws;
+  auto fail = [&](exx_status_t s) {
+    cudaGetLastError();
+    cudaFree(*Gs);
+    cudaFree(*tw);
+    *Gs = *tw = nullptr;
+    b->ws = ws;
+    return s;
+  };
+  *Gs = *tw = nullptr;
+  if (!balloc(b, Gs, gf.size()) || !balloc(b, tw, twf.size() * sizeof(float))) return fail(EXX_ERR_OOM);
   if (cudaMemcpyAsync(*Gs, gf.data(), gf.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
       cudaMemcpyAsync(*tw, twf.data(), twf.size() * sizeof(float), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess) {  // the host buffers die here
-    cudaGetLastError();
-    return EXX_ERR_CUDA;
+      cudaStreamSynchronize(st) != cudaSuccess)  // the host buffers die here
+    return fail(EXX_ERR_CUDA);
+  return EXX_OK;
+}
+
+// What the first enable of the persistent schedule needs: queue segments and,
+// as the queue runs the slab pipeline on the workspace slots of the two pipeline
+// lanes, that pipeline's tables, spectra padded along y and the second slot.
+// Every device allocation goes to `got` until all have succeeded; only then is
+// anything of the batch changed.
+exx_status_t build_queue(exx_batch_t b, cudaStream_t st, std::vector<void*>& got) {
+  got.reserve(2 * b->groups.size() + 8);
+  auto alloc = [&](auto** p, size_t bytes) {
+    if (!balloc(b, p, bytes)) return false;
+    got.push_back(*p);
+    return true;
+  };
+  const char* hook = std::getenv("EXX_TEST_STALL_QUEUE");
+  const bool stall = hook != nullptr && hook[0] == '1';
+  std::vector<QSeg> segs;
+  int mx = 0;
+  for (Group& g : b->groups)
+    if (g.ops->persist_ok) {
+      build_segments(b, g, true, stall, segs);
+      build_segments(b, g, false, stall, segs);
+      mx = std::max(mx, std::max(g.nseg[0], g.nseg[1]));
+    }
+  if (segs.empty()) return EXX_OK;  // no group has a persistent kernel
+  size_t xq = b->x_bytes;
+  std::vector<std::pair<void*, void*>> tab(b->groups.size(), {nullptr, nullptr});
+  for (size_t k = 0; k < b->groups.size(); ++k) {
+    const Group& g = b->groups[k];
+    if (!g.ops->persist_ok) continue;
+    xq = std::max(xq, 2 * g.one);
+    if (!g.plane) continue;
+    const exx_status_t s = group_tables(b, g, false, &tab[k].first, &tab[k].second, st);
+    if (s != EXX_OK) return s;
+    got.push_back(tab[k].first);
+    got.push_back(tab[k].second);
   }
+  const bool slot2 = b->X_2 == nullptr, grow = xq > b->x_bytes;
+  void *x1 = nullptr, *x2 = nullptr, *v2 = nullptr;
+  double* ep2 = nullptr;
+  QSeg* dsegs = nullptr;
+  int* dqc = nullptr;
+  if ((grow && !alloc(&x1, xq)) || ((grow || slot2) && !alloc(&x2, xq)) ||
+      (slot2 && (!alloc(&ep2, b->ep_bytes) || !alloc(&v2, b->v_bytes))) ||
+      !alloc(&dsegs, segs.size() * sizeof(QSeg)) || !alloc(&dqc, (size_t)(mx + 2) * sizeof(int)))
+    return EXX_ERR_OOM;
+  if (cudaMemcpyAsync(dsegs, segs.data(), segs.size() * sizeof(QSeg), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return EXX_ERR_CUDA;
+  if (grow) {  // earlier calls, on whatever stream, still use the spectra that go
+    if (cudaDeviceSynchronize() != cudaSuccess) return EXX_ERR_CUDA;
+    cudaFree(b->X);
+    b->X = x1;
+    b->ws -= b->x_bytes;
+    if (!slot2) {
+      cudaFree(b->X_2);
+      b->ws -= b->x_bytes;
+    }
+    b->x_bytes = xq;
+  }
+  if (grow || slot2) b->X_2 = x2;
+  if (slot2) {
+    b->epart2 = ep2;
+    b->V_2 = v2;
+  }
+  for (size_t k = 0; k < b->groups.size(); ++k)
+    if (tab[k].first != nullptr) {
+      b->groups[k].Gs_q = tab[k].first;
+      b->groups[k].tw_q = tab[k].second;
+    }
+  b->d_segs = dsegs;
+  b->d_qc = dqc;
+  b->qc_len = mx + 2;
+  b->segs.swap(segs);
   return EXX_OK;
 }
 
@@ -781,63 +868,27 @@ exx_status_t exx_batch_set_persistent(exx_batch_t b, int enable, void* cuda_stre
   }
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   if (b->d_segs == nullptr) {
-    const char* hook = std::getenv("EXX_TEST_STALL_QUEUE");
-    const bool stall = hook != nullptr && hook[0] == '1';
-    std::vector<QSeg> segs;
-    int mx = 0;
-    for (Group& g : b->groups)
-      if (g.ops->persist_ok) {
-        build_segments(b, g, true, stall, segs);
-        build_segments(b, g, false, stall, segs);
-        mx = std::max(mx, std::max(g.nseg[0], g.nseg[1]));
-      }
-    if (segs.empty()) return EXX_OK;  // no group has a persistent kernel
-    // the queue runs the slab pipeline on two workspace slots (those of the two
-    // pipeline lanes): its tables, and spectra padded along y
-    size_t xq = b->x_bytes;
-    for (Group& g : b->groups)
-      if (g.ops->persist_ok) {
-        if (g.plane && g.Gs_q == nullptr) {
-          const exx_status_t s = group_tables(b, g, false, &g.Gs_q, &g.tw_q, st);
-          if (s != EXX_OK) return s;
-        }
-        xq = std::max(xq, 2 * g.one);
-      }
-    if (xq > b->x_bytes) {
-      if (cudaStreamSynchronize(st) != cudaSuccess) return EXX_ERR_CUDA;
-      void *x1 = nullptr, *x2 = nullptr;
-      const size_t ws = b->ws;
-      if (!balloc(b, &x1, xq) || (b->X_2 && !balloc(b, &x2, xq))) {
-        if (x1) cudaFree(x1);
-        b->ws = ws;
-        return EXX_ERR_OOM;
-      }
-      cudaFree(b->X);
-      b->X = x1;
-      b->ws -= b->x_bytes;
-      if (b->X_2) {
-        cudaFree(b->X_2);
-        b->X_2 = x2;
-        b->ws -= b->x_bytes;
-      }
-      b->x_bytes = xq;
+    // test hook (EXX_TEST_FAIL_ALLOC=k, k >= 1): the k-th device allocation
+    // reports out of memory without calling cudaMalloc
+    const char* hook = std::getenv("EXX_TEST_FAIL_ALLOC");
+    b->fail_alloc = hook != nullptr ? std::atoi(hook) : 0;
+    b->nalloc = 0;
+    const size_t ws = b->ws;
+    std::vector<void*> got;
+    exx_status_t s;
+    try {
+      s = build_queue(b, st, got);
+    } catch (const std::bad_alloc&) {  // host tables
+      s = EXX_ERR_OOM;
     }
-    if (b->X_2 == nullptr) {
-      if (!balloc(b, &b->epart2, b->ep_bytes) || !balloc(b, &b->X_2, b->x_bytes) ||
-          !balloc(b, &b->V_2, b->v_bytes))
-        return EXX_ERR_OOM;
-    }
-    if (!balloc(b, &b->d_segs, segs.size() * sizeof(QSeg)) ||
-        !balloc(b, &b->d_qc, (size_t)(mx + 2) * sizeof(int)))
-      return EXX_ERR_OOM;
-    b->qc_len = mx + 2;
-    if (cudaMemcpyAsync(b->d_segs, segs.data(), segs.size() * sizeof(QSeg), cudaMemcpyHostToDevice,
-                        st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {
+    b->fail_alloc = 0;
+    if (s != EXX_OK) {
       cudaGetLastError();
-      return EXX_ERR_CUDA;
+      for (void* q : got) cudaFree(q);
+      b->ws = ws;
+      return s;
     }
-    b->segs.swap(segs);
+    if (b->d_segs == nullptr) return EXX_OK;  // no group has a persistent kernel
   }
   for (const Group& g : b->groups)  // function attributes and grid size, outside any capture
     if (g.ops->persist_ok) {
