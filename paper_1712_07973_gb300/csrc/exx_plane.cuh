@@ -274,6 +274,14 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
   constexpr int U2 = YU * SWZ;      // of y forward pass 2 and y inverse pass 1
   constexpr int UZ1 = K::ZUNITS;    // of z passes 1 and 3
   constexpr int UZ2 = ZH * SWR;     // of z pass 2
+  // The tensor-memory instructions are warp-wide (.sync.aligned), and so are the
+  // groups' named barriers: a warp is brought together ahead of them wherever its
+  // lanes may have parted (a last round that not all lanes take, FP64's
+  // left-out twiddles where a warp holds units of two n2); groups hold whole
+  // warps of units.
+  constexpr bool PARTS = UZ1 % NTG != 0 || sizeof(C) == 16;
+  static_assert(K::NG == 1 || (NTG % 32 == 0 && U1 % 32 == 0 && U2 % 32 == 0 && UZ1 % 32 == 0 && UZ2 % 32 == 0 &&
+                               sizeof(C) == 8), "a group's barrier needs whole warps");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* ta_y = reinterpret_cast<C*>(smem_raw);
   C* tb_y = ta_y + Y::L;
@@ -292,6 +300,7 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
   for (int t = tid; t < K::TWN; t += NT) ta_y[t] = tw_g[t];
   unsigned stash = 0;
   if constexpr (!PERZ) {
+    __syncwarp();
     if (warp == 0) tmem_alloc(&tslot, K::tcols);
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   }
@@ -370,6 +379,7 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
             asm volatile("prefetch.global.L2 [%0];\n" ::"l"(nx + t));
         }
       }
+      __syncwarp();
       // z forward, pass 1: units (n2, row), lanes along ky; in place: samples
       // z = ZL2 n1 + n2 become slots ZL2 k1 + n2.  Free lines: the even
       // frequencies first; the samples go to the thread's stash for the odd ones
@@ -385,7 +395,7 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
           for (int n1 = 0; n1 < ZH; ++n1) v[n1] = o[ZL2 * n1];
         }
         if constexpr (!PERZ) {
-          if constexpr (UZ1 % NTG != 0) __syncwarp();
+          if constexpr (PARTS) __syncwarp();
           stash_put(stash + r * K::WST, v);
         }
         if (on) {
@@ -395,7 +405,10 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
           for (int k = 0; k < ZH; ++k) o[ZL2 * k] = v[k];
         }
       }
-      if constexpr (!PERZ) tmem_wait_st();
+      if constexpr (!PERZ) {
+        if constexpr (PARTS) __syncwarp();
+        tmem_wait_st();
+      }
       gsync();
 #pragma unroll 1
       for (int sz = 0; sz < (PERZ ? 1 : 2); ++sz) {
@@ -456,7 +469,7 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
             const int n2 = u / SWR, row = rg + u - n2 * SWR;
             C* o = P + row * ZP + n2;
             C v[ZH], a[ZH];
-            if constexpr (UZ1 % NTG != 0) __syncwarp();
+            if constexpr (PARTS) __syncwarp();
             stash_get(stash + r * K::WST, v);
             if constexpr (!EO) {
               if (on) {
@@ -464,7 +477,7 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
                 for (int k = 0; k < ZH; ++k) a[k] = o[ZL2 * k];
                 dft<ZH, 1, 1>(a);
               }
-              if constexpr (UZ1 % NTG != 0) __syncwarp();
+              if constexpr (PARTS) __syncwarp();
               stash_put(stash + r * K::WST, a);
             }
             if (on) {
@@ -475,7 +488,10 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
               for (int k = 0; k < ZH; ++k) o[ZL2 * k] = v[k];
             }
           }
-          if constexpr (!EO) tmem_wait_st();
+          if constexpr (!EO) {
+            if constexpr (PARTS) __syncwarp();
+            tmem_wait_st();
+          }
           gsync();
         } else if constexpr (!EO) {
           // inverse pass 2 of the odd frequencies, added to the even part
@@ -486,7 +502,7 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
             const int m2 = u / SWR, row = rg + u - m2 * SWR;
             C* o = P + row * ZP + m2;
             C v[ZH], a[ZH];
-            if constexpr (UZ1 % NTG != 0) __syncwarp();
+            if constexpr (PARTS) __syncwarp();
             stash_get(stash + r * K::WST, a);
             if (on) {
 #pragma unroll
