@@ -134,10 +134,11 @@ __host__ __device__ inline void tri_decode(long long g, long long N, int* pi, in
 // ------------------------------------------------- size-independent kernels
 // Per-pair energy: E_ij = h^3 sum of the zconv block partials (one warp per
 // pair, fixed reduction order).
-__global__ void k_pair_energy(const double* __restrict__ epart, int nper,
+__global__ void k_pair_energy(const double* epart_, int nper,
                               const int4* __restrict__ pairs, int npair, double h3,
                               double* __restrict__ Epair) {
   dep_wait();
+  const double* epart = after_wait(epart_);
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= npair) return;
@@ -150,9 +151,10 @@ __global__ void k_pair_energy(const double* __restrict__ epart, int nper,
 
 // E_x = -(alpha/2) sum_{i,j} f_i f_j E_ij = -(alpha/2) sum_{i<=j} (2 - d_ij) f_i f_j E_ij
 // (Eq. HF).  One block, fixed-order tree reduction; pairs decoded on device.
-__global__ void k_exx_total(const double* __restrict__ Epair, long long P, int N,
+__global__ void k_exx_total(const double* Epair_, long long P, int N,
                             const double* __restrict__ occ, double alpha, double* __restrict__ E) {
   dep_wait();
+  const double* Epair = after_wait(Epair_);
   __shared__ double red[256];
   double s = 0.0;
   for (long long g = threadIdx.x; g < P; g += blockDim.x) {
@@ -172,11 +174,12 @@ __global__ void k_exx_total(const double* __restrict__ Epair, long long P, int N
 
 // Both for a call of a single tile (npair = P pairs): the warps take the pairs in
 // turn, then the first 256 threads sum as k_exx_total.
-__global__ void __launch_bounds__(1024) k_pair_energy_total(const double* __restrict__ epart, int nper,
+__global__ void __launch_bounds__(1024) k_pair_energy_total(const double* epart_, int nper,
                                                             const int4* __restrict__ pairs, int npair, double h3,
                                                             double* Epair, int N, const double* __restrict__ occ,
                                                             double alpha, double* __restrict__ E) {
   dep_wait();
+  const double* epart = after_wait(epart_);
   __shared__ double red[256];
   const int lane = threadIdx.x & 31;
   for (int w = threadIdx.x >> 5; w < npair; w += 32) {

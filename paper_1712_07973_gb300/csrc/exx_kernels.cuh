@@ -99,6 +99,15 @@ template <int P, bool FULL, typename C> EXX_HD void dft_inv_out(C* v) {
 // that start earlier and hold their share of an SM while they wait cost 2% at
 // 160^3 and 20% of an FP64 call on 32^3.)
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+// Pointer to what an earlier launch writes, as a value that exists only behind
+// dep_wait: a kernel's const __restrict__ parameter counts as read-only for the
+// whole launch, so its loads might be moved ahead of the wait or take the
+// non-coherent path; none of this one's can.
+template <typename T> __device__ __forceinline__ T* after_wait(T* p) {
+  asm volatile("" : "+l"(p)::"memory");
+  __builtin_assume(__isGlobal(p));
+  return p;
+}
 
 // Tensor-memory-access (TMA) load with an mbarrier (PTX, sm_90 and later).
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
@@ -1038,7 +1047,7 @@ k_accum(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__
   dep_wait();
   const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * VEC;
   if (r >= n3) return;
-  accum_tile<R, TM, VEC, MODE>(psi, V, vx, occ, coef, i0, ti, j0, tj, diag, c, n3, r,
+  accum_tile<R, TM, VEC, MODE>(after_wait(psi), after_wait(V), after_wait(vx), occ, coef, i0, ti, j0, tj, diag, c, n3, r,
                                TOUCH < 0 ? touch : TOUCH, TOUCH < 0 || (TOUCH & T_LAST_I) ? out : nullptr);
 }
 
@@ -1048,10 +1057,13 @@ k_accum(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__
 // twice (from L2).
 template <typename R, int TM, int VEC>
 __global__ void __launch_bounds__(kAccumThreads)
-k_accum_wide(const R* __restrict__ psi, const R* __restrict__ V, double* __restrict__ vx,
+k_accum_wide(const R* psi_, const R* V_, double* vx_,
              const R* __restrict__ occ, const double* __restrict__ coef, int i0, int ti, int j0, int tj, int diag,
              double c, long long n3, int touch, R* out) {
   dep_wait();
+  const R* psi = after_wait(psi_);
+  const R* V = after_wait(V_);
+  double* vx = after_wait(vx_);
   const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * VEC;
   if (r >= n3) return;
   const int s = blockIdx.y;
@@ -1163,7 +1175,7 @@ k_accum_batch(const R* const* __restrict__ psi_tab, const R* __restrict__ V,
               const R* __restrict__ occ, const double* __restrict__ coef, const TileDesc* __restrict__ tiles,
               long long n3) {
   dep_wait();
-  accum_batch_unit<R, TM, VEC, false>(psi_tab, V, vx_tab, vx_out, occ, coef, tiles, n3, blockIdx.x,
+  accum_batch_unit<R, TM, VEC, false>(after_wait(psi_tab), after_wait(V), after_wait(vx_tab), vx_out, occ, coef, tiles, n3, blockIdx.x,
                                       blockIdx.y, blockDim.x);
 }
 

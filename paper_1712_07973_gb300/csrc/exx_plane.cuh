@@ -261,7 +261,7 @@ template <typename R, int G, bool PERY, bool PERZ> struct PlaneBuilt {
 
 template <typename R, int G, bool PERY, bool PERZ, int RY, int NT_, int MINB_, int NG_, bool EO>
 __global__ void __launch_bounds__(NT_, MINB_)
-k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* __restrict__ tw_g,
+k_plane(const cplx<R>* X_, cplx<R>* Yo_, const R* __restrict__ Gs, const cplx<R>* __restrict__ tw_g,
         double* __restrict__ epart, int npair, int nkx) {
   using C = cplx<R>;
   using K = PlaneCfg<R, G, PERY, PERZ, RY, NT_, MINB_, NG_>;
@@ -310,6 +310,8 @@ k_plane(const cplx<R>* X, cplx<R>* Yo, const R* __restrict__ Gs, const cplx<R>* 
     stash = tslot + ((unsigned)(warp & 3) << 21) + (unsigned)(warp >> 2) * (K::ZROUNDS * K::WST);
   }
   dep_wait();
+  const C* X = after_wait(X_);
+  C* Yo = after_wait(Yo_);
   const int nplane = npair * nkx;
   // plane pl: kx = pl / npair, pair pl % npair (the pairs of one kx together:
   // its kernel-table rows stay in L2)
@@ -650,7 +652,7 @@ template <typename R, int N, bool PER> struct XCfg {
 
 template <typename R, int N, bool PER>
 __global__ void __launch_bounds__(XCfg<R, N, PER>::NT, XCfg<R, N, PER>::MINB)
-k_xfwd(const R* __restrict__ psi0, const R* const* __restrict__ psi_tab, const int4* __restrict__ pairs,
+k_xfwd(const R* psi0, const R* const* __restrict__ psi_tab, const int4* __restrict__ pairs,
        cplx<R>* __restrict__ X, const cplx<R>* __restrict__ tw_g, long long n3) {
   using C = cplx<R>;
   using K = XCfg<R, N, PER>;
@@ -665,9 +667,10 @@ k_xfwd(const R* __restrict__ psi0, const R* const* __restrict__ psi_tab, const i
   const int p = blockIdx.x / K::NZB, y = blockIdx.y, z0 = (blockIdx.x - p * K::NZB) * ZB;
   const int4 pr = pairs[p];
   const R* psi = psi_tab ? psi_tab[pr.w] : psi0;
-  const R* __restrict__ pi = psi + (long long)pr.x * n3 + (long long)z0 * G * G + y * G;
-  const R* __restrict__ pj = psi + (long long)pr.y * n3 + (long long)z0 * G * G + y * G;
   dep_wait();
+  psi = after_wait(psi);
+  const R* pi = psi + (long long)pr.x * n3 + (long long)z0 * G * G + y * G;
+  const R* pj = psi + (long long)pr.y * n3 + (long long)z0 * G * G + y * G;
   // rho[2m] + i rho[2m+1], whole rows; paired loads where the caller's orbitals
   // are aligned for them
   if ((reinterpret_cast<size_t>(psi) & (sizeof(C) - 1)) == 0) {
@@ -677,8 +680,8 @@ k_xfwd(const R* __restrict__ psi0, const R* const* __restrict__ psi_tab, const i
     for (int i = 0; i < NL; ++i) {
       const int t = tid + i * NT, zl = t / GC, c = t - zl * GC;
       if (ZB * GC % NT == 0 || t < ZB * GC) {
-        a[i] = __ldg(reinterpret_cast<const C*>(pi + (long long)zl * G * G) + c);
-        b[i] = __ldg(reinterpret_cast<const C*>(pj + (long long)zl * G * G) + c);
+        a[i] = *(reinterpret_cast<const C*>(pi + (long long)zl * G * G) + c);
+        b[i] = *(reinterpret_cast<const C*>(pj + (long long)zl * G * G) + c);
       }
     }
     for (int t = tid; t < 3 * N; t += NT) tw[t] = tw_g[t];
@@ -778,7 +781,7 @@ template <typename C> EXX_HD void fold_step(C xk, C xm, C w, C& zk, C& zm) {
 
 template <typename R, int N, bool PER>
 __global__ void __launch_bounds__(XCfg<R, N, PER>::NT, XCfg<R, N, PER>::MINB)
-k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restrict__ tw_g) {
+k_xinv(const cplx<R>* X, R* __restrict__ V, const cplx<R>* __restrict__ tw_g) {
   using C = cplx<R>;
   using K = XCfg<R, N, PER>;
   constexpr int G = K::G, ZB = K::ZB, X1 = K::X1, X2 = K::X2, SP = K::SP, NT = K::NT;
@@ -788,7 +791,8 @@ k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restri
   C* S = tw + 2 * N;
   const int tid = threadIdx.x;
   const int p = blockIdx.x / K::NZB, y = blockIdx.y, z0 = (blockIdx.x - p * K::NZB) * ZB;
-  const C* Xi = X + ((long long)p * (N + 1) * G + y) * G + z0;
+  dep_wait();
+  const C* Xi = after_wait(X) + ((long long)p * (N + 1) * G + y) * G + z0;
   constexpr int KS = G * G;
   // spectrum side: units (q, zl), zl fastest; the first unit's values are under
   // way during the set-up
@@ -805,7 +809,6 @@ k_xinv(const cplx<R>* __restrict__ X, R* __restrict__ V, const cplx<R>* __restri
     }
     if (q == 0) xn = __ldcs(&in[(long long)N * KS].x);
   };
-  dep_wait();
   if (tid < K::UB) load(tid);
   for (int t = tid; t < 2 * N; t += NT) tw[t] = tw_g[t];
   __syncthreads();
