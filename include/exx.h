@@ -233,16 +233,18 @@ exx_status_t exx_gradient_host(exx_plan_t plan, const void* psi_host, void* grad
 
 /*
  * exx_plan_set_lanes -- number of pipeline lanes (1 to 3) of later calls.
- * A plan is created with two lanes, or one where its slab kernels run as
- * CTA clusters (FP32 n = 160, FP64 n >= 96), or EXX_LANES = 1, 2 or 3
- * from the environment at creation; never more than it has pair tiles; each beyond
- * the first with its own internal stream and spectrum and potential
- * workspaces.  Consecutive tiles go round-robin over the lanes, so the
+ * A plan is created with two lanes, or one where two gain nothing: FP32 free
+ * n = 128 and n = 160, FP64 free n >= 96, wire n = 96 and periodic n = 192; or with
+ * EXX_LANES = 1, 2 or 3 from the environment at creation; never more than it has pair
+ * tiles; each beyond the first with its own internal stream and spectrum and
+ * potential workspaces.  Consecutive tiles go round-robin over the lanes, so the
  * transforms of one tile run beside those of the next; the accumulation stays
  * on the caller's stream in tile order and results are identical bit for bit.
  * One lane serialises every kernel on the caller's stream (per-kernel timing,
  * below, then measures each kernel alone).  Returns EXX_ERR_NOT_SUPPORTED for
- * more lanes than the plan was created with.
+ * more lanes than the plan was created with; an FP32 n = 128 plan without
+ * EXX_LANES also takes two, whose workspaces the first such call allocates
+ * (EXX_ERR_OOM if that fails: the plan goes on with one).
  */
 exx_status_t exx_plan_set_lanes(exx_plan_t plan, int lanes);
 /* exx_plan_get_lanes -- current number of lanes (host out-parameter). */

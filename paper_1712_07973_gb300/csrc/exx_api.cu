@@ -304,9 +304,11 @@ struct exx_plan_s {
   CUtensorMap gmap{};      // TMA descriptor of the kernel table (Ops::stage_table)
   void* h_psi = nullptr;  // exx_apply_host staging (allocated on first use)
   void* h_vx = nullptr;
-  // pipeline lanes (run): lanes in use, lanes with workspaces, and the
-  // workspaces, streams and events of lanes 1.. (lane 0 uses X2, V, epart)
-  int lanes = 1, max_lanes = 1;
+  // pipeline lanes (run): lanes in use, lanes that may be asked for, lanes with
+  // workspaces, and the workspaces, streams and events of lanes 1.. (lane 0 uses
+  // X2, V, epart; a plan of one lane has no streams)
+  int lanes = 1, max_lanes = 1, have_lanes = 1;
+  size_t x_bytes = 0, v_bytes = 0, ep_bytes = 0;
   void* X2x[kMaxLanes] = {};
   void* Vx[kMaxLanes] = {};
   double* epx[kMaxLanes] = {};
@@ -403,6 +405,25 @@ template <typename T> exx_status_t dalloc(exx_plan_t p, T** out, size_t bytes) {
   }
   p->ws += bytes;
   *out = static_cast<T*>(q);
+  return EXX_OK;
+}
+
+// Workspaces, streams and events for `lanes` pipeline lanes.  Synchronous; a
+// failure keeps what was made (used by the next call, freed with the plan).
+exx_status_t make_lanes(exx_plan_t p, int lanes) {
+  exx_status_t s;
+  for (int l = 1; l < lanes; ++l)
+    if ((p->epx[l] == nullptr && (s = dalloc(p, &p->epx[l], p->ep_bytes)) != EXX_OK) ||
+        (p->X2x[l] == nullptr && (s = dalloc(p, &p->X2x[l], p->x_bytes)) != EXX_OK) ||
+        (p->Vx[l] == nullptr && (s = dalloc(p, &p->Vx[l], p->v_bytes)) != EXX_OK))
+      return s;
+  for (int l = 0; lanes > 1 && l < lanes; ++l) {
+    if (p->ls[l] == nullptr) EXX_CUDA(p, cudaStreamCreateWithFlags(&p->ls[l], cudaStreamNonBlocking));
+    if (p->ev_done[l] == nullptr) EXX_CUDA(p, cudaEventCreateWithFlags(&p->ev_done[l], cudaEventDisableTiming));
+    if (p->ev_free[l] == nullptr) EXX_CUDA(p, cudaEventCreateWithFlags(&p->ev_free[l], cudaEventDisableTiming));
+  }
+  if (lanes > 1 && p->ev_fork == nullptr) EXX_CUDA(p, cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
+  p->have_lanes = std::max(p->have_lanes, lanes);
   return EXX_OK;
 }
 
@@ -652,10 +673,13 @@ static exx_status_t plan_create_impl(exx_plan_t* out, const int grid[3], const d
   EXX_ALLOC(p->d_occ, norb * (2 * sizeof(double) + sizeof(float)));
   p->d_occf = reinterpret_cast<float*>(p->d_occ + 2 * (size_t)norb);
   EXX_ALLOC(p->d_pairs, pairs.size() * sizeof(int4));
-  EXX_ALLOC(p->epart, (size_t)p->maxpairs * nper * sizeof(double));
+  p->ep_bytes = (size_t)p->maxpairs * nper * sizeof(double);
+  p->x_bytes = xbytes;
+  p->v_bytes = (size_t)p->maxpairs * n3 * rs;
+  EXX_ALLOC(p->epart, p->ep_bytes);
   EXX_ALLOC(p->Epair, (size_t)p->P * sizeof(double));
   EXX_ALLOC(p->X2, xbytes);
-  EXX_ALLOC(p->V, (size_t)p->maxpairs * n3 * rs);
+  EXX_ALLOC(p->V, p->v_bytes);
   if (precision == EXX_FP32 && !(flags & EXX_FLAG_VX_FP64)) {
     EXX_ALLOC(p->vacc, (size_t)norb * n3 * sizeof(double));
   }
@@ -665,18 +689,21 @@ static exx_status_t plan_create_impl(exx_plan_t* out, const int grid[3], const d
   // beside the other tile's plane kernel: 96^3 8.33 -> 8.15 ms with 32
   // orbitals), one where the planes go through in halves (160^3 24 orbitals 25.7
   // ms with one lane, 26.4 with two; 128^3 12.5 and 12.65) or the slab kernels run
-  // as CTA clusters; EXX_LANES=1..3 at plan creation chooses; never more than the
-  // plan has tiles
+  // as CTA clusters; the workspaces of a second lane that is not the default (128^3) are
+  // made when exx_plan_set_lanes asks for it; EXX_LANES=1..3 at plan creation
+  // chooses; never more than the plan has tiles
   {
     const char* env = std::getenv("EXX_LANES");
-    int nl = (p->plane ? ops->plane_ry == 2 : ops->clustered) ? 1 : kDefaultLanes;
-    if (env && env[0] >= '1' && env[0] <= '0' + kMaxLanes && env[1] == '\0') nl = env[0] - '0';
-    p->max_lanes = p->lanes = (int)std::min<size_t>((size_t)nl, p->tiles.size());
+    int nl = (p->plane ? ops->plane_ry == 2 : ops->clustered) ? 1 : kDefaultLanes, most = ops->clustered ? nl : kDefaultLanes;
+    if (env && env[0] >= '1' && env[0] <= '0' + kMaxLanes && env[1] == '\0') nl = most = env[0] - '0';
+    p->lanes = (int)std::min<size_t>((size_t)nl, p->tiles.size());
+    p->max_lanes = (int)std::min<size_t>((size_t)most, p->tiles.size());
   }
-  for (int l = 1; l < p->max_lanes; ++l) {
-    EXX_ALLOC(p->epx[l], (size_t)p->maxpairs * nper * sizeof(double));
-    EXX_ALLOC(p->X2x[l], xbytes);
-    EXX_ALLOC(p->Vx[l], (size_t)p->maxpairs * n3 * rs);
+  if ((st_ = make_lanes(p, p->lanes)) != EXX_OK) {
+    cudaGetLastError();
+    free_plan(p);
+    delete p;
+    return st_;
   }
 #undef EXX_ALLOC
 
@@ -711,14 +738,6 @@ static exx_status_t plan_create_impl(exx_plan_t* out, const int grid[3], const d
   if (e == cudaSuccess && ops->stage_table && !p->plane && !exx::make_ktab_map(&p->gmap, p->Gs, nh, nz))
     e = cudaErrorInvalidValue;
   if (e == cudaSuccess) e = p->plane ? ops->plane_setup() : ops->setup();
-  if (e == cudaSuccess && p->max_lanes > 1) {
-    for (int l = 0; l < p->max_lanes && e == cudaSuccess; ++l) {
-      e = cudaStreamCreateWithFlags(&p->ls[l], cudaStreamNonBlocking);
-      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_done[l], cudaEventDisableTiming);
-      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_free[l], cudaEventDisableTiming);
-    }
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming);
-  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     free_plan(p);
@@ -1056,6 +1075,10 @@ exx_status_t exx_gradient_host(exx_plan_t p, const void* psi_host, void* grad_ho
 exx_status_t exx_plan_set_lanes(exx_plan_t p, int lanes) {
   if (p == nullptr || lanes < 1 || lanes > kMaxLanes) return EXX_ERR_INVALID_ARG;
   if (lanes > p->max_lanes) return EXX_ERR_NOT_SUPPORTED;
+  if (lanes > p->have_lanes) {
+    const exx_status_t s = make_lanes(p, lanes);
+    if (s != EXX_OK) return s;
+  }
   p->lanes = lanes;
   return EXX_OK;
 }
