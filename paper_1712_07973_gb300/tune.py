@@ -4,8 +4,8 @@ The tile edge T (orbitals per tile side, 1..8) trades the amortisation of the
 orbital reads and FP64 accumulator updates (which fall as 1/T per pair) against
 the size of each launch and of the workspace (T^2 pairs per tile).  ``tune``
 times exx_apply for a few candidates on seeded orbitals of the requested size
-and keeps the fastest in a JSON cache keyed by (n, N, precision, SM count);
-``best_tile`` reads it.  The cache path is $EXX_TUNE_CACHE, else
+and keeps the fastest (the larger of those that the timing cannot tell apart) in
+a JSON cache keyed by (n, N, precision, SM count); ``best_tile`` reads it.  The cache path is $EXX_TUNE_CACHE, else
 ~/.cache/exx_gb300/tiles.json.
 """
 
@@ -65,15 +65,18 @@ def best_tile(n, N, precision="fp32", tune_if_missing=False, path=None):
     return 0
 
 
-# timings this close are ties: small molecules are bound by their launches, whose
-# times scatter by a few per cent from one process to the next
-TIE = 0.10
+# Timings (ms) this close are ties.  Short calls are bound by their launches, whose
+# times scatter by a few microseconds from one run to the next (six processes, 18
+# timings each: 4.4 us of 42 at 16^3 with 10 orbitals, 4.3 of 72 at 24^3 with 16, 7.9 of
+# 69 at 32^3 with 12); a call of milliseconds repeats to 0.3% (96^3, 24 orbitals),
+# where this is 0.13% and the fastest is taken.
+TIE_MS = 0.006
 
 
 def select(timings):
-    """Fastest candidate; ties (within TIE of the fastest) go to the larger tile
-    (less accumulator traffic)."""
-    most = (1.0 + TIE) * min(timings.values())
+    """Fastest candidate; ties (within TIE_MS of the fastest) go to the larger
+    tile (less accumulator traffic)."""
+    most = min(timings.values()) + TIE_MS
     return max(t for t in timings if timings[t] <= most)
 
 
@@ -108,6 +111,7 @@ def _gpu_measure(n, N, precision, h, reps):
     def measure(tile):
         plan = exx.ExxPlan(n, h, 0.25, occ, precision=precision, tile=tile)
         out = torch.empty(psi.shape, dtype=plan.vx_dtype, device=psi.device)
+
         def timed(calls):
             a = torch.cuda.Event(enable_timing=True)
             b = torch.cuda.Event(enable_timing=True)
