@@ -5,7 +5,8 @@ orbital reads and FP64 accumulator updates (which fall as 1/T per pair) against
 the size of each launch and of the workspace (T^2 pairs per tile).  ``tune``
 times exx_apply for a few candidates on seeded orbitals of the requested size
 and keeps the fastest (the larger of those that the timing cannot tell apart) in
-a JSON cache keyed by (n, N, precision, SM count); ``best_tile`` reads it.  The cache path is $EXX_TUNE_CACHE, else
+a JSON cache keyed by (n, N, precision, SM count); ``best_tile`` reads it, but
+for entries timed on other kernels (KERNELS).  The cache path is $EXX_TUNE_CACHE, else
 ~/.cache/exx_gb300/tiles.json.
 """
 
@@ -15,6 +16,9 @@ import os
 __all__ = ["CANDIDATES", "cache_path", "cache_key", "load_cache", "store", "best_tile", "tune"]
 
 CANDIDATES = (2, 4, 6, 8)
+# the kernels that cached timings hold for: raised when the pipeline's change
+# (entries without it: the slab pipeline on every grid)
+KERNELS = "plane-1"
 
 
 def cache_path():
@@ -41,7 +45,7 @@ def load_cache(path=None):
 def store(key, tile, timings, path=None):
     path = path or cache_path()
     d = load_cache(path)
-    d[key] = {"tile": int(tile), "ms": {str(k): float(v) for k, v in timings.items()}}
+    d[key] = {"tile": int(tile), "kernels": KERNELS, "ms": {str(k): float(v) for k, v in timings.items()}}
     os.makedirs(os.path.dirname(path) or ".", exist_ok=True)
     tmp = path + ".tmp"
     with open(tmp, "w") as fh:
@@ -58,7 +62,7 @@ def best_tile(n, N, precision="fp32", tune_if_missing=False, path=None):
     """Cached tile edge for (n, N, precision) on this GPU, or 0 (library default)."""
     key = cache_key(n, N, precision, _sm_count())
     e = load_cache(path).get(key)
-    if e:
+    if e and e.get("kernels") == KERNELS:
         return int(e["tile"])
     if tune_if_missing:
         return tune(n, N, precision, path=path)[0]

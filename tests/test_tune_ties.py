@@ -1,4 +1,6 @@
-"""Which timings the tile tuner takes as ties (no GPU)."""
+"""Which timings the tile tuner takes as ties, and which cached ones it trusts (no GPU)."""
+
+import json
 
 import pytest
 
@@ -14,3 +16,18 @@ from paper_1712_07973_gb300 import tune
 ])
 def test_ties_are_the_scatter_of_short_calls(timings, best):
     assert tune.select(timings) == best
+
+
+def test_tiles_timed_on_other_kernels_are_not_reused(tmp_path, monkeypatch):
+    path = str(tmp_path / "tiles.json")
+    monkeypatch.setattr(tune, "_sm_count", lambda: 152)
+    key = tune.cache_key(96, 64, "fp32", 152)
+    with open(path, "w") as fh:  # as written before entries named their kernels
+        json.dump({key: {"tile": 4, "ms": {"4": 1.0, "8": 2.0}}}, fh)
+    assert tune.best_tile(96, 64, "fp32", path=path) == 0
+    tune.tune(96, 64, "fp32", path=path, measure=lambda t: 9.0 - t, sm_count=152)
+    assert tune.best_tile(96, 64, "fp32", path=path) == 8
+    d = json.load(open(path))
+    d[key]["kernels"] = "other"
+    json.dump(d, open(path, "w"))
+    assert tune.best_tile(96, 64, "fp32", path=path) == 0
