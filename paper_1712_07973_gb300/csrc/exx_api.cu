@@ -132,16 +132,11 @@ __host__ __device__ inline void tri_decode(long long g, long long N, int* pi, in
 }
 
 // ------------------------------------------------- size-independent kernels
-// Per-pair energy: E_ij = h^3 sum of the zconv block partials (one warp per
-// pair, fixed reduction order).
-__global__ void k_pair_energy(const double* epart_, int nper,
-                              const int4* __restrict__ pairs, int npair, double h3,
-                              double* __restrict__ Epair) {
-  dep_wait();
-  const double* epart = after_wait(epart_);
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+// Pair w's energy by one warp: E_ij = h^3 sum of the plane kernel's (zconv's)
+// partials, in a fixed reduction order.
+__device__ __forceinline__ void pair_energy(const double* epart, int nper, const int4* __restrict__ pairs, int w,
+                                            double h3, double* Epair) {
   const int lane = threadIdx.x & 31;
-  if (w >= npair) return;
   double s = 0.0;
   for (int t = lane; t < nper; t += 32) s += epart[(long long)w * nper + t];
 #pragma unroll
@@ -150,49 +145,14 @@ __global__ void k_pair_energy(const double* epart_, int nper,
 }
 
 // E_x = -(alpha/2) sum_{i,j} f_i f_j E_ij = -(alpha/2) sum_{i<=j} (2 - d_ij) f_i f_j E_ij
-// (Eq. HF).  One block, fixed-order tree reduction; pairs decoded on device.
-__global__ void k_exx_total(const double* Epair_, long long P, int N,
-                            const double* __restrict__ occ, double alpha, double* __restrict__ E) {
-  dep_wait();
-  const double* Epair = after_wait(Epair_);
+// (Eq. HF) by the first 256 threads of a block, fixed-order tree reduction;
+// pairs decoded on device.
+__device__ __forceinline__ void exx_total(const double* Epair, long long P, int N, const double* __restrict__ occ,
+                                          double alpha, double* E) {
   __shared__ double red[256];
-  double s = 0.0;
-  for (long long g = threadIdx.x; g < P; g += blockDim.x) {
-    int i, j;
-    tri_decode(g, N, &i, &j);
-    const double m = (i == j) ? 1.0 : 2.0;
-    s += m * occ[i] * occ[j] * Epair[g];
-  }
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *E = -0.5 * alpha * red[0];
-}
-
-// Both for a call of a single tile (npair = P pairs): the warps take the pairs in
-// turn, then the first 256 threads sum as k_exx_total.
-__global__ void __launch_bounds__(1024) k_pair_energy_total(const double* epart_, int nper,
-                                                            const int4* __restrict__ pairs, int npair, double h3,
-                                                            double* Epair, int N, const double* __restrict__ occ,
-                                                            double alpha, double* __restrict__ E) {
-  dep_wait();
-  const double* epart = after_wait(epart_);
-  __shared__ double red[256];
-  const int lane = threadIdx.x & 31;
-  for (int w = threadIdx.x >> 5; w < npair; w += 32) {
-    double s = 0.0;
-    for (int t = lane; t < nper; t += 32) s += epart[(long long)w * nper + t];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) Epair[pairs[w].z] = h3 * s;
-  }
-  __syncthreads();
   if (threadIdx.x < 256) {
     double s = 0.0;
-    for (long long g = threadIdx.x; g < npair; g += 256) {
+    for (long long g = threadIdx.x; g < P; g += 256) {
       int i, j;
       tri_decode(g, N, &i, &j);
       const double m = (i == j) ? 1.0 : 2.0;
@@ -206,6 +166,34 @@ __global__ void __launch_bounds__(1024) k_pair_energy_total(const double* epart_
     __syncthreads();
   }
   if (threadIdx.x == 0) *E = -0.5 * alpha * red[0];
+}
+
+// One warp per pair.
+__global__ void k_pair_energy(const double* epart, int nper, const int4* __restrict__ pairs, int npair, double h3,
+                              double* __restrict__ Epair) {
+  dep_wait();
+  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w < npair) pair_energy(after_wait(epart), nper, pairs, w, h3, Epair);
+}
+
+// One block of 256.
+__global__ void k_exx_total(const double* Epair, long long P, int N, const double* __restrict__ occ, double alpha,
+                            double* __restrict__ E) {
+  dep_wait();
+  exx_total(after_wait(Epair), P, N, occ, alpha, E);
+}
+
+// Both for a call of a single tile (npair = P pairs): the warps of one block of
+// 1024 take the pairs in turn.
+__global__ void __launch_bounds__(1024) k_pair_energy_total(const double* epart, int nper,
+                                                            const int4* __restrict__ pairs, int npair, double h3,
+                                                            double* Epair, int N, const double* __restrict__ occ,
+                                                            double alpha, double* __restrict__ E) {
+  dep_wait();
+  epart = after_wait(epart);
+  for (int w = threadIdx.x >> 5; w < npair; w += 32) pair_energy(epart, nper, pairs, w, h3, Epair);
+  __syncthreads();
+  exx_total(Epair, npair, N, occ, alpha, E);
 }
 
 __global__ void k_to_float(const double* __restrict__ a, float* __restrict__ b, long long n) {

@@ -30,8 +30,7 @@ bool kernel_spectrum_octant(int n, double h, int kind, double omega, double* out
 
 namespace exx {
 const Ops* find_ops(int prec, int n);
-__global__ void k_pair_energy(const double* __restrict__ epart, int nper,
-                              const int4* __restrict__ pairs, int npair, double h3,
+__global__ void k_pair_energy(const double* epart, int nper, const int4* __restrict__ pairs, int npair, double h3,
                               double* __restrict__ Epair);
 
 struct MolTot {
