@@ -200,9 +200,12 @@ def pipeline_bytes(n, N, T, rs=4, bc="free"):
     grids the plane pipeline is not built for; else, the kinds standing for
     xfwd, plane and xinv, the same with the spectrum unpadded ((h+1) n n
     complex), and with an orbital's first accumulation not read and its last
-    one written as the FP32 output."""
+    one written as the output.  Minimal: planes that go through in halves (FP32
+    free 128^3 and 160^3, FP64 free 96^3 and 112^3) are read twice by their kernel
+    and their partial outputs once, mostly from L2, which is not counted."""
     tot = algorithmic_bytes(n, N, T, rs, bc)
-    if n < 16 or n > (128 if bc == "periodic" else 160):
+    most = {"periodic": (128, 96), "free": (160, 112)}.get(bc, (96, 96))[0 if rs == 4 else 1]
+    if n < 16 or n > most:
         return tot
     hl, _ = half_lines(n, bc)
     less = (hl + 1) * n * (2 * hl - n) * 2 * rs  # padding of one pair's spectrum

@@ -253,7 +253,10 @@ exx_status_t exx_plan_get_lanes(exx_plan_t plan, int* lanes);
 /*
  * Per-kernel timing with CUDA events recorded on the launching stream around
  * every launch of the pipeline (kernel kinds, in order: 0 fwd_xy, 1 zconv,
- * 2 pair_energy, 3 inv_yx, 4 accum, 5 exx_total, 6 to_float).
+ * 2 pair_energy, 3 inv_yx, 4 accum, 5 exx_total, 6 to_float).  Where the plane
+ * pipeline runs, kinds 0, 1 and 3 are its x transforms, its (y, z) plane kernel
+ * and its inverse x transforms; a call of one tile times its pair energies and
+ * total under kind 5; kind 6 runs in sharded and overlapping calls only.
  * exx_profile_enable(plan, 1) starts recording (0 stops); exx_profile_read
  * synchronises on the recorded events and returns, per kind, the summed
  * milliseconds (host ms[EXX_NKINDS]) and launch counts (host
@@ -360,12 +363,15 @@ exx_status_t exx_batch_graph(exx_batch_t batch, int enable);
  * tiles from a device work queue, instead of five launches per wave.  Items of
  * a pass wait (bounded, on the device) for the items they depend on: a wait
  * that runs out sets the flag that exx_batch_pair_energies reports as
- * EXX_ERR_TIMEOUT, and the rest of the launch is skipped.  Results equal those
- * of the launch-per-pass schedule bit for bit.  FP32 grids whose slab kernels
+ * EXX_ERR_TIMEOUT, and the rest of the launch is skipped.  The queue runs the
+ * slab kernels on every grid, where the launch-per-pass schedule runs the plane
+ * pipeline from n = 16: results of the two agree to FP32 rounding (1e-6 Ha), and
+ * each is bit-identical from call to call.  FP32 grids whose slab kernels
  * run as CTA clusters (n = 160) keep the launch-per-pass schedule.  The first
- * enable builds the queue tables, allocates a second workspace slot if the
- * batch has none (returns EXX_ERR_OOM if that fails) and synchronises the
- * stream; it discards captured graphs.
+ * enable builds the queue's kernel tables and segments, allocates its spectra
+ * and a second workspace slot if the batch has none, and synchronises the
+ * device; if it fails (EXX_ERR_OOM) the batch stays as it was.  Every enable
+ * discards captured graphs.
  */
 exx_status_t exx_batch_set_persistent(exx_batch_t batch, int enable, void* cuda_stream);
 

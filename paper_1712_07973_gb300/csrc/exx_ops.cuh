@@ -324,20 +324,18 @@ template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> stru
   static constexpr int QA = SA.q, NT_A = SA.nt, MINB_A = SA.minb, CL_A = SA.cl;
   static constexpr int QC = SC.q, NT_C = SC.nt, MINB_C = SC.minb, CL_C = SC.cl;
   static constexpr size_t smem_a = SA.smem, smem_c = SC.smem;
-  // FP32 z lines of L2 = 6 (96 points: periodic and wire 96^3, free 48^3): six
-  // warps, so that each pass-1 and pass-3 unit has its own warp, and six CTAs
-  // per SM (periodic 96^3 -3.3%, wire -9% per exx_apply against 12 warps)
-  // (FP32 L2 = 14, 224-point lines: eight warps, two rounds in every pass,
-  // rather than seven with three rounds in the second; FP32 L2 = 12,
-  // 192-point lines: eight warps with the kernel table read from L2, four
-  // CTAs per SM, -2.3% zconv at 96^3 against twelve warps with the staged
-  // table at three CTAs)
-  // (FP32 320-point lines of free 160^3, split 20 x 16 (split_z): ten warps, two
-  // CTAs per SM; 16 columns per CTA with two units per warp, five warps and
-  // four CTAs per SM, measured 7% slower)
+  // zconv's CTA.  In FP32 it runs the allocation-free entry point's energies (free
+  // grids up to 96^3), grids below 16 points and periodic 192^3; the figures are from
+  // when it ran the grids they name, most of which the plane pipeline took over.
+  // L2 = 6 (96-point z lines): six warps, so that each pass-1 and pass-3 unit has
+  // its own warp, and six CTAs per SM (periodic 96^3 -3.3%, wire -9% per exx_apply
+  // against 12 warps).  L2 = 12 (192 points): eight warps with the kernel table
+  // read from L2, four CTAs per SM (-2.3% zconv at 96^3 against twelve warps with the
+  // staged table at three CTAs).  320 points, split 20 x 16 (split_z): ten warps,
+  // two CTAs per SM (16 columns per CTA with two units per warp, five warps and
+  // four CTAs per SM, measured 7% slower); no FP32 grid launches that one now.
   static constexpr int NW = (sizeof(R) == 4 && LZ1 == 20)   ? 10  // 320-point lines (split_z)
                             : (sizeof(R) == 4 && LZ2 == 6)  ? 6
-                            : (sizeof(R) == 4 && LZ2 == 14) ? 8
                             : (sizeof(R) == 4 && LZ2 == 12) ? 8
                                                             : zconv_warps(LZ2);
   static constexpr int W = L < 32 ? L : 32;
@@ -398,8 +396,8 @@ template <typename R, int N, bool PER = false, int NZ = N, bool PERZ = PER> stru
     return cudaErrorNotSupported;
   }
 
-  // plane pipeline: every grid of 16 points and more whose spectrum plane, or
-  // half of it, fits an SM (FP32 up to 160^3 free and 128^3 periodic, FP64 up to
+  // plane pipeline: every even grid of 16 points and more whose spectrum plane,
+  // or half of it, fits an SM (FP32 up to 160^3 free and 128^3 periodic, FP64 up to
   // 112^3 and 96^3).  Against the slab pipeline per call (FP32, two lanes): 96^3
   // 32 orbitals 9.98 -> 8.50 ms, 160^3 32 orbitals 60.6 -> 46.6, 64^3 16 orbitals
   // 0.782 -> 0.673, periodic 96^3 32 orbitals 3.96 -> 3.63; 16^3 4 orbitals 41.1 ->

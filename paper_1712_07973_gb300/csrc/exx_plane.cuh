@@ -13,11 +13,14 @@
 //
 // The padded (y, z) part of a spectrum never reaches memory: per pair X (8 n^3
 // bytes in FP32) is written and read twice, where spectra X[kx][z][ky] padded
-// along y move twice that four times.
+// along y move twice that four times.  Planes that go through in halves (128^3,
+// 160^3) are read once more and their partial outputs written and read once more
+// by the plane kernel, most of that in L2: at 160^3 it moves 47 MB in and 41 out per
+// pair, its spectrum being 33.
 //
 // What bounds it, per pair in FP32 (HBM at 6.8 TB/s, the FMA pipe, shared memory at
-// 128 bytes a cycle and SM; measured): plane 96^3 2.1, 6.1, 6.8; 9.9 us (start: 8.2
-// for z alone, 17.5 with the y passes of the slab kernels), 160^3 9.7, 34, 32; 59 us.
+// 128 bytes a cycle and SM; measured): plane 96^3 2.1, 6.1, 6.8; 9.9 us (slab pipeline:
+// 8.2 for z alone, 17.5 with the y passes of its kernels), 160^3 9.7, 34, 32; 59 us.
 // xfwd 96^3 1.0 us of HBM, 1.9 measured; 160^3 4.9 and 9.0 (exchange through shared
 // memory 60% busy).  xinv 96^3 1.6 and 1.9; 160^3 7.3 and 8.2.
 #pragma once
@@ -170,8 +173,8 @@ template <int H, typename C> __device__ __forceinline__ void stash_get(unsigned 
 }
 
 // -------------------------------------------------------------------- plane
-// Shared memory, the FMA pipe and instruction issue are each about 65% busy; HBM
-// 20%.  Hence: every pass in place (the plane is all the shared memory there
+// Shared memory is 78% busy at 96^3 and 66% at 160^3, the FMA pipe and instruction
+// issue 56 to 59%, HBM 20%.  Hence: every pass in place (the plane is all the shared memory there
 // is), odd pitch and lanes across lines (no bank conflicts, warp-uniform
 // twiddles read two at a time), barriers of groups rather than of the CTA, and
 // the z samples and partial outputs in tensor memory rather than a second half

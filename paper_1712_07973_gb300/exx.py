@@ -325,11 +325,14 @@ class ExxPlan:
                                           _stream_ptr(stream)), "exx_gradient_host", self.handle)
         return E.value
 
+    # kernel kinds of profile_read; the plane pipeline's x transforms, plane kernel
+    # and inverse x transforms count as fwd_xy, zconv and inv_yx
     KINDS = ("fwd_xy", "zconv", "pair_energy", "inv_yx", "accum", "exx_total", "to_float")
 
     def set_lanes(self, lanes):
         """1: every kernel on the caller's stream; 2: consecutive tiles on two
-        internal streams (the default where the plan has several tiles)."""
+        internal streams (the default where the plan has several tiles and two
+        lanes gain something: exx_plan_set_lanes in include/exx.h)."""
         _check(self.lib.exx_plan_set_lanes(self.handle, int(lanes)), "exx_plan_set_lanes", self.handle)
 
     def profile(self, enable=True):
