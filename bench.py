@@ -47,7 +47,7 @@ sys.path.insert(0, ROOT)
 WORKLOAD = "c5_large_n160_N512"
 METRIC = "EXX pair-solves/s and ms per E_x+gradient: FP32 batched vs FP64 plain at ≤1e-6 Ha"
 UNIT = "pair-solves/s"
-KERNEL_SOURCES = ["exx_fft.cuh", "exx_kernels.cuh", "exx_ops.cuh"]
+KERNEL_SOURCES = ["exx_fft.cuh", "exx_kernels.cuh", "exx_ops.cuh", "exx_plane.cuh"]
 WORKLOADS = ["c5_large_n160_N512", "c3_grad_n128_N128", "c2_fp32_n96_N64"]
 
 

@@ -968,8 +968,10 @@ enum Touch { T_FIRST_I = 1, T_FIRST_J = 2, T_LAST_I = 4 };
 // coef = null: the exchange action, vx_k += c * sum; else the gradient of E_x,
 // vx_k += coef_k * sum, coef_k = -alpha 2 h^3 f_k (dE_x/dpsi_k = 2 f_k h^3 (Vx
 // psi)_k, Eq. daction), the per-orbital factor folded into the FP64
-// accumulation.  occ: the occupations in the working precision.  (Forming both
-// per thread, and converting the sums on the FP64 units, kept those 66% busy.)
+// accumulation.  occ: the occupations in the working precision.  (Tables rather
+// than formed per thread, and sums widened by integer instructions: 0.68 -> 0.55 us
+// per pair at 56^3, 1.82 -> 1.77 at 96^3.  The FP64 pipe is still 66% active at 96^3
+// and 76% at 160^3 where a tile is an orbital's first and last.)
 // touch: Touch bits; out: the output that takes an orbital's last update.
 template <typename R, int TM, int VEC, int MODE, bool COH = false>
 __device__ __forceinline__ void accum_tile(const R* __restrict__ psi, const R* __restrict__ V,
@@ -1037,7 +1039,7 @@ __device__ __forceinline__ void accum_tile(const R* __restrict__ psi, const R* _
 // given by touch.
 // CTAs of 128 threads, the registers of 512 (768 in the ragged form) per SM; with
 // the potentials marked evict-first: full FP32 tiles 0.66 -> 0.58 us per pair at
-// 64^3, 1.94 -> 1.85 at 96^3 (4.3 TB/s), 8.4 -> 8.0 at 160^3.
+// 64^3, 1.94 -> 1.85 at 96^3, 8.4 -> 8.0 at 160^3; with what followed 1.73 and 7.5.
 constexpr int kAccumThreads = 128;
 template <typename R, int TM, int VEC, int MODE, int TOUCH>
 __global__ void __launch_bounds__(kAccumThreads, (sizeof(R) == 4 && MODE == 0) ? 6 : 4)
